@@ -578,7 +578,7 @@ back_kernel(BackParams<T> P)
                 // lists of this group or found by walking the tree; one copy of
                 // the step's code serves both (the kernel's code stays small)
                 const uint32_t ln = P.list_n ? P.list_n[g] : kListOverflow;
-                const bool replay = ln != kListOverflow;
+                const bool replay = ln <= (uint32_t)P.list_K;
                 const uint32_t* ids = P.list_ids + (int64_t)g * P.list_K;
                 int nf = 0, sp = 1;
                 uint32_t base = 0;

@@ -8,6 +8,7 @@
 // evaluation differs.  psi is Neumaier-compensated like the other outputs.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "potential.cuh"
 #include "walk_dev.cuh"
@@ -66,23 +67,28 @@ LENS_DEV float2 ein_poly2(float2 u)
 template <int KIND, typename T, int R> struct PsiCtx {
     using value_type = T;
     using Buf = WalkBuf<KIND, T>;
-    static constexpr int kKind = KIND;
+    static constexpr int kKind = KIND, kR = R;
+    static constexpr bool kCuts = true;
     static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
     const WalkParams<T>& P;
     const PsiConsts<T> K;
     WalkBuf<KIND, T>* B;
     WalkRanges* Rg;
+    WalkCut* Cut;
     v2_t<T> H;
     vec4_t<T> box;
+    // boxes visited, cells accepted, leaf particles, big entries scanned, kept
+    uint32_t c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0;
     int nf = 0, nn = 0, nb = 0;
     uint32_t* rec = nullptr;  // (the potential keeps no interaction lists)
+    uint32_t* rec_shared = nullptr;
     int rec_n = 0, rec_cap = 0;
     T lx[R], ly[R];
     T part[R][3];              // psi, alpha1, alpha2 of the current flush
     T tot_s[R][3], tot_c[R][3];  // compensated totals
 
     LENS_DEV PsiCtx(const WalkParams<T>& p, const PsiConsts<T>& k, WalkShared<KIND, T>& s)
-        : P(p), K(k), B(&s.buf), Rg(&s.rng) {}
+        : P(p), K(k), B(&s.buf), Rg(&s.rng), Cut(&s.cut) {}
 
     LENS_DEV void zero()
     {
@@ -352,9 +358,15 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
     bool rv[R];
     for (;;) {
         uint32_t g = 0;
-        if (lane == 0) g = atomicAdd(P.counter, 1u);
-        g = __shfl_sync(full, g, 0);
-        if ((int64_t)g >= P.n_groups) break;
+        if constexpr (DIRECT) {
+            if (lane == 0) g = atomicAdd(P.counter, 1u);
+            g = __shfl_sync(full, g, 0);
+            if ((int64_t)g >= P.n_groups) break;
+        } else {
+            if (!next_item(P, stack, S.cut)) break;
+            g = S.cut.g;
+        }
+        const bool head = DIRECT || S.cut.item == kNoItem;  // the group's first (or only) item
         C.H = P.gH[g];
         C.box = P.gbox[g];
         const uint2 rg = P.grange[g];
@@ -373,43 +385,46 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
                 ridx[r] = 0;
             }
         }
-        C.zero();
         C.nf = C.nn = C.nb = 0;
-        int c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0, c_dummy = 0;
-        if (P.n_part > 0) {
-            if (DIRECT) {
+        C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
+        if constexpr (DIRECT) {
+            C.zero();
+            if (P.n_part > 0) {
                 for (int64_t base = 0; base < P.n_part; base += 0x40000000) {
                     const int64_t rem = P.n_part - base;
                     const int c = (int)(rem < 0x40000000 ? rem : 0x40000000);
-                    append_ranges(C, lane == 0 ? c : 0, (int)base, P.leaf0, P.leaf1, c_near, c_dummy);
+                    append_ranges(C, lane == 0 ? c : 0, (int)base, P.leaf0, P.leaf1);
                 }
                 C.flush_near();
-            } else {
-                traverse(C, stack, c_vis, c_acc, c_near, c_bigs, c_bigk);
+            }
+            if (P.n_halos > 0) C.halos();
+        } else {
+            do {  // (once, or once for each part of a cut whose pool was full)
+                C.zero();
+                traverse(C, stack, S.cut.sp);
                 C.flush_far();
                 C.flush_near();
                 C.flush_big();
-            }
+                if (P.n_halos > 0 && head && S.cut.seg == 0) C.halos();
+            } while (S.cut.local && local_next_part<R, 3>(P.cut, S.cut, stack, [&](int r, int q) {
+                         return C.tot_s[r][q] + C.tot_c[r][q]; }));
         }
-        if (P.n_halos > 0) C.halos();
-        if (P.stats && lane == 0) {
-            const unsigned long long nr = rg.y;
-            atomicAdd(&P.stats[0], 1ull);
-            atomicAdd(&P.stats[1], (unsigned long long)c_vis);
-            atomicAdd(&P.stats[2], (unsigned long long)c_acc);
-            atomicAdd(&P.stats[3], (unsigned long long)c_near);
-            atomicAdd(&P.stats[4], (unsigned long long)c_bigs);
-            atomicAdd(&P.stats[5], (unsigned long long)c_bigk);
-            atomicAdd(&P.stats[6], nr * (unsigned long long)(c_acc + c_near + c_bigk));
-        }
+        __syncwarp();
+        count_item(C, g, rg.y, head);
+        T* tot = DIRECT ? nullptr : item_totals<R>(P.cut, S.cut);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            if (!rv[r]) continue;
+            if (!rv[r] && !tot) continue;
             const uint32_t i = ridx[r];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                if (!P.out[q]) continue;
                 T val = C.tot_s[r][q] + C.tot_c[r][q];
+                if (!DIRECT && S.cut.local) val = local_total<R>(P.cut, r, q);
+                if (tot) {
+                    tot[(q * R + r) * 32 + lane] = val;
+                    continue;
+                }
+                if (!P.out[q]) continue;
                 if (P.accumulate) val += P.out[q][i];
                 P.out[q][i] = val;
             }
@@ -429,7 +444,8 @@ static void psi_launch_one(const WalkParams<T>& P, const PsiConsts<T>& K, int nu
                                  (int)smem);
         int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psi_kernel<KIND, T, R, DIRECT>, kWalkWarps * 32, smem);
-        bps = std::min(std::max(nb, 1), 16);  // stacks are allocated for 16 blocks per SM
+        // stacks are allocated for 16 blocks per SM, a tree walk's cut slots for kCutBlocks
+        bps = std::min(std::max(nb, 1), DIRECT ? 16 : kCutBlocks);
     }
     { psi_kernel<KIND, T, R, DIRECT><<<num_sms * bps, kWalkWarps * 32, smem, s>>>(P, K); note_launch(); }
 }
@@ -503,15 +519,22 @@ static lens_status psi_typed(lens_tree* t, const ShootPlan& plan, const void* dx
     bool first = true;
     int launches = 0;
     auto launch = [&](int kind, const PsiConsts<T>& K) {
-        P.counter = counter + 2 * launches;
-        cudaMemsetAsync(P.counter, 0, sizeof(uint32_t), s);
+        P.counter = counter + 8 * launches;
+        cudaMemsetAsync(P.counter, 0, 8 * sizeof(uint32_t), s);
         if (plan.n == 0) return;
-        if (plan.R == 1) {
-            if (direct) psi_launch_kind<T, 1, true>(kind, P, K, t->num_sms, s);
-            else psi_launch_kind<T, 1, false>(kind, P, K, t->num_sms, s);
+        const int64_t ng = (int64_t)plan.ng;
+        // (a lens without particles has nothing to walk: the direct form)
+        if (direct || P.n_part == 0) {
+            if (plan.R == 1) psi_launch_kind<T, 1, true>(kind, P, K, t->num_sms, s);
+            else psi_launch_kind<T, 2, true>(kind, P, K, t->num_sms, s);
         } else {
-            if (direct) psi_launch_kind<T, 2, true>(kind, P, K, t->num_sms, s);
-            else psi_launch_kind<T, 2, false>(kind, P, K, t->num_sms, s);
+            auto go = [&](auto rays) {
+                constexpr int R = decltype(rays)::value;
+                auto walk = [&](const WalkParams<T>& Q) { psi_launch_kind<T, R, false>(kind, Q, K, t->num_sms, s); };
+                walk_rounds<T, R>(P, ng, 3, base, L, P.counter, walk, s);
+            };
+            if (plan.R == 1) go(std::integral_constant<int, 1>{});
+            else go(std::integral_constant<int, 2>{});
         }
     };
     for (const SpeciesTree& st : t->sp) {

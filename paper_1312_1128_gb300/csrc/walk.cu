@@ -23,6 +23,7 @@
 // against its correction when a ray passes close to a listed particle.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "profiles.cuh"
 #include "sort.cuh"
@@ -99,6 +100,18 @@ __global__ void k_bbox_init(unsigned long long* bbox, int64_t nb)
     bbox[4 * b + 3] = 0ull;
 }
 
+// Order-preserving map of a float to uint32.
+__device__ __forceinline__ uint32_t flt_to_ordered(float f)
+{
+    uint32_t u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float ordered_to_flt(uint32_t u)
+{
+    u = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
+    return __uint_as_float(u);
+}
+
 __device__ __forceinline__ uint32_t spread16(uint32_t x)
 {
     x &= 0xffffu;
@@ -128,11 +141,22 @@ __global__ void k_ray_keys(const int64_t* boff, int nb, const double* borig, con
     vals[i] = (uint32_t)i;
 }
 
+// Mark group g if its box is stretched (kStretch): ex, ey = half sides of an
+// even share of its batch.
+template <typename T>
+__device__ __forceinline__ void mark_stretched(int64_t g, T hx, T hy, T ex, T ey, uint8_t* gflag, uint32_t* sub)
+{
+    const bool st = (hx > T(kStretch) * ex && hx > T(1e-25)) || (hy > T(kStretch) * ey && hy > T(1e-25));
+    gflag[g] = st ? 1 : 0;
+    if (st) sub[16 + atomicAdd(sub, 1u)] = (uint32_t)g;
+}
+
 template <typename T, int R>
 __global__ void k_groups(int64_t n_groups, const int64_t* boff, const uint32_t* gfirst, int nb,
                          const double* borig, const void* dx, const void* dy, int dtype,
                          const uint32_t* svals, v2_t<T>* gH, vec4_t<T>* gbox, uint2* grange,
-                         v2_t<T>* ray_l, uint32_t* ray_idx)
+                         v2_t<T>* ray_l, uint32_t* ray_idx, const unsigned long long* bbox, const uint32_t* bb32,
+                         uint8_t* gflag, uint32_t* sub)
 {
     const unsigned full = 0xffffffffu;
     int lane = threadIdx.x & 31;
@@ -217,6 +241,16 @@ __global__ void k_groups(int64_t n_groups, const int64_t* boff, const uint32_t* 
         bx.x = cx; bx.y = cy; bx.z = hx; bx.w = hy;
         gbox[g] = bx;
         grange[g] = make_uint2((uint32_t)first, (uint32_t)count);
+        const float share = 0.5f * sqrtf((float)GR / (float)(boff[b + 1] - boff[b]));
+        float wx, wy;
+        if (bb32) {
+            wx = ordered_to_flt(bb32[2]) - ordered_to_flt(bb32[0]);
+            wy = ordered_to_flt(bb32[3]) - ordered_to_flt(bb32[1]);
+        } else {
+            wx = (float)(ordered_to_dbl(bbox[4 * b + 1]) - ordered_to_dbl(bbox[4 * b]));
+            wy = (float)(ordered_to_dbl(bbox[4 * b + 3]) - ordered_to_dbl(bbox[4 * b + 2]));
+        }
+        mark_stretched<T>(g, hx, hy, (T)(wx * share), (T)(wy * share), gflag, sub);
     }
 }
 
@@ -226,17 +260,6 @@ __global__ void k_groups(int64_t n_groups, const int64_t* boff, const uint32_t* 
 // the offsets (relative positions do not depend on the origin), and, when
 // the origin is zero, groups anchored at H = 0 with l = the offsets
 // themselves -- what the FP64 path computes in that case.
-__device__ __forceinline__ uint32_t flt_to_ordered(float f)
-{
-    uint32_t u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float ordered_to_flt(uint32_t u)
-{
-    u = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
-    return __uint_as_float(u);
-}
-
 // bb = {min x, min y, max x, max y} as ordered images; the caller sets the
 // minima to 0xffffffff and the maxima to 0 first.
 __global__ void __launch_bounds__(256) k_ray_bbox32(const float* dx, const float* dy, int64_t n, uint32_t* bb)
@@ -291,7 +314,8 @@ __global__ void k_ray_keys32(const float* dx, const float* dy, int64_t n, const 
 // T, so H = 0 and l = the offset (as k_groups then has it).
 template <typename T, int R>
 __global__ void k_groups32(int64_t n_groups, int64_t n, const float* dx, const float* dy, const uint32_t* svals,
-                           v2_t<T>* gH, vec4_t<T>* gbox, uint2* grange, v2_t<T>* ray_l, uint32_t* ray_idx)
+                           v2_t<T>* gH, vec4_t<T>* gbox, uint2* grange, v2_t<T>* ray_l, uint32_t* ray_idx,
+                           const uint32_t* bb32, uint8_t* gflag, uint32_t* sub)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -332,14 +356,19 @@ __global__ void k_groups32(int64_t n_groups, int64_t n, const float* dx, const f
         bx.x = cx; bx.y = cy; bx.z = hx; bx.w = hy;
         gbox[g] = bx;
         grange[g] = make_uint2((uint32_t)first, (uint32_t)count);
+        const float share = 0.5f * sqrtf((float)(32 * R) / (float)n);
+        mark_stretched<T>(g, hx, hy, (T)((ordered_to_flt(bb32[2]) - ordered_to_flt(bb32[0])) * share),
+                          (T)((ordered_to_flt(bb32[3]) - ordered_to_flt(bb32[1])) * share), gflag, sub);
     }
 }
 
 // ---------------------------------------------------------------- walk
 
-template <int KIND, typename T, int R, bool AO, bool DIRECT, int TILE>
-__global__ void __launch_bounds__(kWalkWarps * 32, sizeof(T) == 4 ? (R == 4 ? 4 : (R == 2 ? 5 : 6)) : 2)
-walk_kernel(WalkParams<T> P)
+// LOC: with local expansions (local.cuh).  FP32 NFW trees, and point masses
+// where the groups are many enough for supergroups (launch_super).
+template <int KIND, typename T, int R, bool AO, bool DIRECT, int TILE, bool LOC>
+__global__ void __launch_bounds__(kWalkWarps * 32, sizeof(T) == 4 ? (LOC || R == 4 ? 4 : (R == 2 ? 4 : 5)) : 2)
+walk_kernel(const __grid_constant__ WalkParams<T> P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned full = 0xffffffffu;
@@ -347,27 +376,130 @@ walk_kernel(WalkParams<T> P)
     using WS = WalkShared<KIND, T, TILE, tot_rays<R>()>;
     WS& S = reinterpret_cast<WS*>(smem_raw)[warp];
     int* stack = P.stack + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
-    WalkCtx<KIND, T, R, AO, TILE> C(P, S);
-    uint32_t ridx[R];
-    bool rv[R];
+    using Ctx = WalkCtx<KIND, T, R, AO, TILE, LOC>;
+    Ctx C(P, S);
 
     const int NS = DIRECT && P.n_slices > 1 ? P.n_slices : 1;
+    for (;;) {
+        uint32_t slice = 0, g = 0;
+        if constexpr (DIRECT) {
+            uint32_t item = 0;
+            if (lane == 0) item = atomicAdd(P.counter, 1u);
+            item = __shfl_sync(full, item, 0);
+            if ((int64_t)item >= P.n_groups * NS) break;
+            slice = item % (uint32_t)NS;
+            g = item / (uint32_t)NS;
+        } else {
+            if (!next_item(P, stack, S.cut)) break;
+            g = S.cut.g;
+        }
+        // the group's first (or only) item
+        const bool head = DIRECT ? slice == 0 : S.cut.item == kNoItem;
+        C.load_group(g);
+        if constexpr (DIRECT) {
+            C.start();
+            if (KIND >= 0 && P.n_part > 0) {
+                // every particle of this item's slice with its full profile
+                const int64_t p0 = P.n_part * slice / NS, p1 = P.n_part * (slice + 1) / NS;
+                for (int64_t base = p0; base < p1; base += 0x40000000) {
+                    int64_t rem = p1 - base;
+                    int c = (int)(rem < 0x40000000 ? rem : 0x40000000);
+                    append_ranges(C, lane == 0 ? c : 0, (int)base, P.leaf0, P.leaf1);
+                }
+                C.flush_near();
+            }
+            if (P.n_halos > 0 && head) Ctx::Flush::finish(P.halos, P.n_halos, nullptr, float4{});
+        } else {
+            C.rec = P.list_ids ? P.list_ids + (int64_t)g * P.list_K : nullptr;
+            C.rec_shared = head ? nullptr : P.list_n + g;
+            C.rec_n = 0;
+            C.rec_cap = P.list_K;
+            do {  // (once, or once for each part of a cut whose pool was full)
+                C.start();
+                const bool whole = traverse(C, stack, S.cut.sp);
+                if (C.rec && lane == 0) {
+                    // (above the room, whatever parts add to it: the lists did not fit)
+                    if (head) P.list_n[g] = whole && C.rec_n <= C.rec_cap && (S.cut.seg == 0 || P.list_n[g] != kListTooLong)
+                                                ? (uint32_t)C.rec_n : kListTooLong;
+                    else if (!whole) atomicOr(P.list_n + g, kListTooLong);
+                }
+                C.flush_far();
+                C.flush_near();
+                C.flush_big();
+                const bool first = head && S.cut.seg == 0;
+                const SuperRec* sr = nullptr;
+                float4 delta = make_float4(0.f, 0.f, 0.f, 0.f);
+                if constexpr (LOC) {
+                    if (P.super && first && P.super[g / kSuperGroups].ok == 1) {
+                        sr = P.super + g / kSuperGroups;
+                        delta = P.sdelta[g];
+                    }
+                }
+                Ctx::Flush::finish(P.halos, first ? P.n_halos : 0, sr, delta);
+            } while (S.cut.local && local_next_part<R, AO ? 2 : 5>(P.cut, S.cut, stack,
+                                                                   [&](int r, int q) { return C.total(r, q); }));
+        }
+        __syncwarp();
+        const uint2 rg = P.grange[g];
+        count_item(C, g, rg.y, head);
+
+        T* tot = DIRECT ? nullptr : item_totals<R>(P.cut, S.cut);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int k = r * 32 + lane;
+            const bool ray = k < (int)rg.y;
+            if (!ray && !tot) continue;
+            const uint32_t i = ray ? P.ray_idx[rg.x + k] : 0u;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                if (AO && q >= 2) break;
+                T val = C.total(r, q);
+                if (!DIRECT && S.cut.local) val = local_total<R>(P.cut, r, q);
+                if (NS > 1) {
+                    P.split[((int64_t)slice * 5 + q) * P.split_n + i] = val;
+                    continue;
+                }
+                if (tot) {
+                    tot[(q * R + r) * 32 + lane] = val;
+                    continue;
+                }
+                if (P.accumulate) val += P.out[q][i];
+                P.out[q][i] = val;
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// The plain tree walk: whole groups, with P.skip all but the stretched ones.
+template <int KIND, typename T, int R, bool AO, int TILE>
+__global__ void __launch_bounds__(kWalkWarps * 32, sizeof(T) == 4 ? (R == 4 ? 4 : (R == 2 ? 5 : 6)) : 2)
+walk_plain(const __grid_constant__ WalkParams<T> P)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const unsigned full = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    PlainShared<KIND, T, TILE, tot_rays<R>()>& S = reinterpret_cast<PlainShared<KIND, T, TILE, tot_rays<R>()>*>(smem_raw)[warp];
+    int* stack = P.stack + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
+    PlainCtx<KIND, T, R, AO, TILE> C(P, &S.buf, &S.tot, &S.rng);
+    uint32_t ridx[R];
+    bool rv[R];
     for (;;) {
         uint32_t item = 0;
         if (lane == 0) item = atomicAdd(P.counter, 1u);
         item = __shfl_sync(full, item, 0);
-        if ((int64_t)item >= P.n_groups * NS) break;
-        const uint32_t slice = item % (uint32_t)NS;
-        const uint32_t g = P.order ? P.order[item / (uint32_t)NS] : item / (uint32_t)NS;
+        if ((int64_t)item >= P.n_groups) break;
+        const uint32_t g = P.order ? P.order[item] : item;
+        if (P.skip && P.gflag[g]) continue;
         C.H = P.gH[g];
         C.box = P.gbox[g];
-        uint2 rg = P.grange[g];
+        const uint2 rg = P.grange[g];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            int k = r * 32 + lane;
+            const int k = r * 32 + lane;
             rv[r] = k < (int)rg.y;
             if (rv[r]) {
-                v2_t<T> l = P.ray_l[rg.x + k];
+                const v2_t<T> l = P.ray_l[rg.x + k];
                 C.lx[r] = l.x;
                 C.ly[r] = l.y;
                 ridx[r] = P.ray_idx[rg.x + k];
@@ -379,62 +511,345 @@ walk_kernel(WalkParams<T> P)
             C.part[r].zero();
         }
         C.tot_zero();
-
-        int c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0, c_dummy = 0;
+        C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
         C.nf = C.nn = C.nb = 0;
-        if (KIND >= 0 && P.n_part > 0) {
-            if (DIRECT) {
-                // every particle of this item's slice with its full profile
-                const int64_t p0 = P.n_part * slice / NS, p1 = P.n_part * (slice + 1) / NS;
-                for (int64_t base = p0; base < p1; base += 0x40000000) {
-                    int64_t rem = p1 - base;
-                    int c = (int)(rem < 0x40000000 ? rem : 0x40000000);
-                    append_ranges(C, lane == 0 ? c : 0, (int)base, P.leaf0, P.leaf1, c_near, c_dummy);
-                }
-                C.flush_near();
-            } else {
-                C.rec = P.list_ids ? P.list_ids + (int64_t)g * P.list_K : nullptr;
-                C.rec_n = 0;
-                C.rec_cap = P.list_K;
-                const bool whole = traverse(C, stack, c_vis, c_acc, c_near, c_bigs, c_bigk);
-                if (C.rec && lane == 0)
-                    P.list_n[g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListOverflow;
-                C.flush_far();
-                C.flush_near();
-                if constexpr (KIND != LENS_POINT) C.flush_big();
-            }
-        }
-        if (P.n_halos > 0 && slice == 0) C.halos();
-        if (P.gcost && lane == 0) P.gcost[g] += (uint32_t)(c_vis + c_acc + c_near + c_bigk);
-        if (P.stats && lane == 0) {
-            unsigned long long nr = rg.y;
-            if (slice == 0) atomicAdd(&P.stats[0], 1ull);
-            atomicAdd(&P.stats[1], (unsigned long long)c_vis);
-            atomicAdd(&P.stats[2], (unsigned long long)c_acc);
-            atomicAdd(&P.stats[3], (unsigned long long)c_near);
-            atomicAdd(&P.stats[4], (unsigned long long)c_bigs);
-            atomicAdd(&P.stats[5], (unsigned long long)c_bigk);
-            atomicAdd(&P.stats[6], nr * (unsigned long long)(c_acc + c_near + c_bigk));
-        }
-
+        C.rec = P.list_ids ? P.list_ids + (int64_t)g * P.list_K : nullptr;
+        C.rec_n = 0;
+        C.rec_cap = P.list_K;
+        if (lane == 0) stack[0] = 0;
+        __syncwarp();
+        const bool whole = traverse(C, stack, 1);
+        if (C.rec && lane == 0)
+            P.list_n[g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListTooLong;
+        C.flush_far();
+        C.flush_near();
+        if constexpr (KIND != LENS_POINT) C.flush_big();
+        if (P.n_halos > 0) C.halos(P.halos, P.n_halos);
+        count_item(C, g, rg.y, true);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (!rv[r]) continue;
-            uint32_t i = ridx[r];
+            const uint32_t i = ridx[r];
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
                 if (AO && q >= 2) break;
                 T val = C.tot_get(r, q);
-                if (NS > 1) {
-                    P.split[((int64_t)slice * 5 + q) * P.split_n + i] = val;
-                    continue;
-                }
                 if (P.accumulate) val += P.out[q][i];
                 P.out[q][i] = val;
             }
         }
         __syncwarp();
     }
+}
+
+template <int KIND, typename T, int R, bool AO, int TILE>
+static void launch_plain(const WalkParams<T>& P, int num_sms, cudaStream_t s)
+{
+    constexpr size_t smem = kWalkWarps * sizeof(PlainShared<KIND, T, TILE, tot_rays<R>()>);
+    static const int bps = [] {
+        if (smem > 48 * 1024)
+            cudaFuncSetAttribute(walk_plain<KIND, T, R, AO, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(walk_plain<KIND, T, R, AO, TILE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        int nb = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, walk_plain<KIND, T, R, AO, TILE>, kWalkWarps * 32, smem);
+        return std::min(std::max(nb, 1), 16);  // stack slots are allocated for 16 blocks per SM
+    }();
+    walk_plain<KIND, T, R, AO, TILE><<<num_sms * bps, kWalkWarps * 32, smem, s>>>(P);
+    note_launch();
+}
+
+// The common part of the walk of kSuperGroups consecutive groups of a point-
+// mass tree (SuperRec), one warp each, one group per lane.
+//
+// The warp walks the tree as the first group's own walk does: the same tests,
+// the same order, the same buffers, evaluated at the groups' centres.  Beside
+// the first group's test every box gets two bounds: it is accepted for all if
+// the supergroup's box is beyond r_cut, opened for all if the box's farthest
+// point is within (a margin of 1e-5 covers the rounding of the groups' own
+// tests).  Accepted for all and far from the supergroup, or a leaf opened for
+// all and far: its sources go to the expansion.  Any other box that is not
+// opened for all is left to the groups; what the first group's walk finds
+// inside it (kLeftBit) is evaluated in its place and taken off again at the
+// end.  More boxes left than a record holds: the groups start at the root.
+// (A walk of more than kSuperWork boxes and entries is that of a stretched
+// group: not worth one warp's time.)
+constexpr uint32_t kSuperWork = 16384;
+constexpr int kSuperLeft = 128, kTinyLeft = 8;      // most boxes left to the groups
+constexpr float kNarrow = 0.01f, kTiny = 1e-6f;     // of the root's r_cm
+static_assert(kSuperLeft <= kCutNodes, "room in the record");
+constexpr int kLeftBit = 1 << 30;  // (a tree has fewer boxes)
+
+__global__ void __launch_bounds__(kWalkWarps * 32, 4)
+k_super(const __grid_constant__ WalkParams<float> P, const float* rcm, const unsigned long long* bbox,
+        const uint32_t* bb32, SuperRec* rec, float4* sdelta)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    using Flush = WalkFlush<LENS_POINT, float, 1, false, 0, true>;
+    using WS = Flush::WS;
+    const unsigned full = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    WS& S = reinterpret_cast<WS*>(smem_raw)[warp];
+    uint8_t* far_left = S.loc.idx;             // of the far buffer's cells and the
+    uint8_t* near_left = S.loc.idx + kBigCap;  // near buffer's particles: left to the groups
+    int* stack = P.stack + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
+    const int64_t n_super = (P.n_groups + kSuperGroups - 1) / kSuperGroups;
+    // One batch over a patch small against the lens: a tiny one, where all
+    // rays of a group share the rounding of their sums, with few boxes left; or
+    // no expansions at all (every ray's sum then keeps its own order, SuperRec).
+    float ext = INFINITY;
+    if (bb32)
+        ext = fmaxf(ordered_to_flt(bb32[2]) - ordered_to_flt(bb32[0]), ordered_to_flt(bb32[3]) - ordered_to_flt(bb32[1]));
+    else if (bbox)
+        ext = (float)fmax(ordered_to_dbl(bbox[1]) - ordered_to_dbl(bbox[0]),
+                             ordered_to_dbl(bbox[3]) - ordered_to_dbl(bbox[2]));
+    const bool narrow = ext < kNarrow * rcm[0];
+    const int most_left = !narrow ? kSuperLeft : ext < kTiny * rcm[0] ? kTinyLeft : -1;
+    for (;;) {
+        uint32_t sg = 0;
+        if (lane == 0) sg = atomicAdd(P.counter, 1u);
+        sg = __shfl_sync(full, sg, 0);
+        if ((int64_t)sg >= n_super) break;
+        SuperRec& Q = rec[sg];
+        const int64_t g = (int64_t)sg * kSuperGroups + lane;
+        const bool have = g < P.n_groups;
+        const float2 Hg = P.gH[have ? g : (int64_t)sg * kSuperGroups];
+        const float4 bg = P.gbox[have ? g : (int64_t)sg * kSuperGroups];
+        const float Hx = __shfl_sync(full, Hg.x, 0), Hy = __shfl_sync(full, Hg.y, 0);
+        const float4 b0 = make_float4(__shfl_sync(full, bg.x, 0), __shfl_sync(full, bg.y, 0),
+                                      __shfl_sync(full, bg.z, 0), __shfl_sync(full, bg.w, 0));
+        const float gx = (Hg.x - Hx) + bg.x, gy = (Hg.y - Hy) + bg.y;  // this group's centre
+        float x0 = gx - bg.z, x1 = gx + bg.z, y0 = gy - bg.w, y1 = gy + bg.w;
+        for (int o = 16; o; o >>= 1) {
+            x0 = fminf(x0, __shfl_xor_sync(full, x0, o));
+            x1 = fmaxf(x1, __shfl_xor_sync(full, x1, o));
+            y0 = fminf(y0, __shfl_xor_sync(full, y0, o));
+            y1 = fmaxf(y1, __shfl_xor_sync(full, y1, o));
+        }
+        const float cx = 0.5f * (x0 + x1), cy = 0.5f * (y0 + y1);
+        const float hx = fmaxf(x1 - cx, cx - x0) * 1.00001f, hy = fmaxf(y1 - cy, cy - y0) * 1.00001f;
+        const float d = box_radius(hx, hy), far2 = d * d * (1.0f / kLocRho2);
+        if (lane == 0) stack[0] = 0;
+        local_zero(S.loc.sum);
+        __syncwarp();
+        LocalH L;
+        L.zero();
+        // alpha at this group's centre, and of it what is left to the groups;
+        // gamma without what is left (a star at the centre would drown it)
+        Comp5<float> all, own;
+        all.zero();
+        own.zero();
+        float top2 = 0.0f;  // largest |alpha|^2 of one star left to the groups
+        int sp = 1, left = 0, nf = 0, nn = 0;
+        uint32_t work = 0;
+        bool ok = d < 1e30f;
+        // The buffers hold positions as the tree has them: the sums at the
+        // centres subtract each group's own anchor, as its own walk does (the
+        // subtraction is rounded: the anchor is part of the result's last digits).
+        auto flush_far = [&]() {
+            Acc5<float> a, f;
+            a.zero();
+            f.zero();
+            for (int b = 0; b < nf; b += 32) {
+                const unsigned m = __ballot_sync(full, b + lane < nf && far_left[b + lane]);
+                const int e = nf - b < 32 ? nf - b : 32;
+                for (int j = 0; j < e; ++j) {
+                    const int i = b + j;
+                    const float wx = bg.x - (S.buf.fdx[i] - Hg.x), wy = bg.y - (S.buf.fdy[i] - Hg.y);
+                    if (m >> j & 1u) {
+                        cell_terms<float, true>(f, wx, wy, S.buf.fM[i], S.buf.fqr[i], S.buf.fqi[i]);
+                        cell_terms<float, true>(a, wx, wy, S.buf.fM[i], S.buf.fqr[i], S.buf.fqi[i]);
+                    } else {
+                        cell_terms<float, false>(f, wx, wy, S.buf.fM[i], S.buf.fqr[i], S.buf.fqi[i]);
+                    }
+                }
+            }
+            all.add(f);
+            own.add(a);
+            for (int i = lane; i < nf; i += 32) {
+                if (far_left[i]) continue;
+                const float wx = cx - (S.buf.fdx[i] - Hx), wy = cy - (S.buf.fdy[i] - Hy);
+                L.cell(wx, wy, rcp(fmaf(wx, wx, wy * wy)), d, S.buf.fM[i], S.buf.fqr[i], S.buf.fqi[i]);
+            }
+            __syncwarp();
+            nf = 0;
+        };
+        auto flush_near = [&]() {
+            Acc5<float> a, f;
+            a.zero();
+            f.zero();
+            for (int b = 0; b < nn; b += 32) {
+                const unsigned m = __ballot_sync(full, b + lane < nn && near_left[b + lane]);
+                const int e = nn - b < 32 ? nn - b : 32;
+                for (int j = 0; j < e; ++j) {
+                    const float4 q = S.buf.n0[b + j];
+                    const float wx = bg.x - (q.x - Hg.x), wy = bg.y - (q.y - Hg.y);
+                    float kb, Dp;
+                    point_terms(q.z, fmaf(wx, wx, wy * wy), kb, Dp);
+                    if (m >> j & 1u) {
+                        f.radial<true>(wx, wy, kb, 0.0f, Dp);
+                        a.radial<true>(wx, wy, kb, 0.0f, Dp);
+                        top2 = fmaxf(top2, kb * kb * fmaf(wx, wx, wy * wy));
+                    } else {
+                        f.radial<false>(wx, wy, kb, 0.0f, Dp);
+                    }
+                }
+            }
+            all.add(f);
+            own.add(a);
+            for (int i = lane; i < nn; i += 32) {
+                if (near_left[i]) continue;
+                const float4 q = S.buf.n0[i];
+                const float wx = cx - (q.x - Hx), wy = cy - (q.y - Hy);
+                L.point(wx, wy, rcp(fmaf(wx, wx, wy * wy)), d, q.z);
+            }
+            __syncwarp();
+            nn = 0;
+        };
+        while (sp > 0 && ok) {
+            const int k = sp < 32 ? sp : 32;
+            sp -= k;
+            const int e = lane < k ? stack[sp + lane] : -1;
+            __syncwarp();
+            const int v = e & (kLeftBit - 1);
+            bool acc = false, leaf = false, open = false, is_left = false, keep = false;
+            float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
+            int4 Lk = make_int4(0, 0, 0, 0);
+            float dx = 0.f, dy = 0.f;
+            if (e >= 0) {
+                A = P.nodeA[v];
+                Lk = P.link[v];
+                dx = A.x - Hx;
+                dy = A.y - Hy;
+                // the first group's test
+                const float ex = fmaxf(fabsf(dx - b0.x) - b0.z, 0.0f), ey = fmaxf(fabsf(dy - b0.y) - b0.w, 0.0f);
+                acc = fmaf(ex, ex, ey * ey) > A.w;
+                leaf = !acc && (Lk.y & kLeafBit);
+                open = !acc && !leaf;
+                is_left = (e & kLeftBit) != 0;
+                if (!is_left) {
+                    const float ux = fabsf(dx - cx), uy = fabsf(dy - cy);
+                    const float lx = fmaxf(ux - hx, 0.0f), ly = fmaxf(uy - hy, 0.0f);
+                    const float fx = ux + hx, fy = uy + hy;
+                    const float w2 = fmaf(ux, ux, uy * uy);
+                    const bool all_acc = fmaf(lx, lx, ly * ly) > A.w * 1.00001f;
+                    const bool all_opn = fmaf(fx, fx, fy * fy) * 1.00001f < A.w;
+                    // every particle of a leaf is within r_cm of its centre of mass
+                    const float m = sqrtf(w2) - rcm[v] * 1.00001f;
+                    keep = acc ? !(all_acc && w2 >= far2) : leaf ? !(all_opn && m > 0.0f && m * m >= far2) : !all_opn;
+                    is_left = keep;
+                }
+            }
+            const unsigned lt = (1u << lane) - 1u;
+            unsigned ball = __ballot_sync(full, acc);
+            if (acc) {
+                const int pos = nf + __popc(ball & lt);
+                const float2 Qm = P.nodeB[v];
+                S.buf.fdx[pos] = A.x;
+                S.buf.fdy[pos] = A.y;
+                S.buf.fM[pos] = A.z;
+                S.buf.fqr[pos] = Qm.x;
+                S.buf.fqi[pos] = Qm.y;
+                far_left[pos] = is_left ? 1 : 0;
+            }
+            nf += __popc(ball);
+            work += (uint32_t)(k + __popc(ball));
+            ball = __ballot_sync(full, keep);
+            if (left + __popc(ball) > most_left) {
+                ok = false;
+                break;
+            }
+            if (keep) Q.nodes[left + __popc(ball & lt)] = v;
+            left += __popc(ball);
+            const int nc = open ? Lk.y : 0;
+            int totc;
+            const int offc = warp_exclusive_scan(nc, &totc);
+            if (sp + totc > kStackCap) {
+                if (lane == 0) atomicOr(P.err, DERR_STACK_OVERFLOW);
+                ok = false;
+                break;
+            }
+            for (int c = 0; c < nc; ++c) stack[sp + offc + c] = (Lk.x + c) | (is_left ? kLeftBit : 0);
+            sp += totc;
+            // leaf particles, in order, as append_ranges takes them
+            const int cnt = leaf ? (Lk.y & kCountMask) : 0;
+            int tot;
+            const int off = warp_exclusive_scan(cnt, &tot);
+            work += (uint32_t)tot;
+            for (int b = 0; b < tot; b += 32) {
+                if (nn + 32 > kNearCap) flush_near();
+                for (int c = 0; c < cnt; ++c) {
+                    const int i = off + c - b;
+                    if (i < 0 || i >= 32) continue;
+                    S.buf.n0[nn + i] = P.leaf0[Lk.x + c];
+                    near_left[nn + i] = is_left ? 1 : 0;
+                }
+                nn += tot - b < 32 ? tot - b : 32;
+                __syncwarp();
+            }
+            __syncwarp();
+            if (nf >= 32) flush_far();
+            ok = work < kSuperWork;
+        }
+        if (ok) {
+            flush_far();
+            flush_near();
+            Flush::add_h(L);
+            LocalFields& F = *reinterpret_cast<LocalFields*>(S.buf.n0);
+            local_finish(S.loc.sum, F);
+            const float id = 1.0f / d;
+            Acc5<float> a;
+            a.zero();
+            local_eval<false>(F, (gx - cx) * id, (gy - cy) * id, id, a);
+            if (have) {
+                const float e[5] = {a.a1, a.a2, 0.0f, a.g1, a.g2};
+                float v[5];
+#pragma unroll
+                for (int q = 0; q < 5; ++q)
+                    v[q] = ((all.s[q] - own.s[q]) - e[q]) + (all.c[q] - own.c[q]);
+                // where one star outweighs the rest (it lies at the centre), the
+                // difference of alpha is that star's rounding
+                if (sqrtf(top2) > 0.5f * (fabsf(all.s[0]) + fabsf(all.s[1]))) v[0] = v[1] = 0.0f;
+                const float4 dl = make_float4(v[0], v[1], v[3], v[4]);
+                sdelta[g] = dl;
+                if (P.gcost) atomicAdd(P.gcost + g, work);
+            }
+            if (lane < kLocH) Q.h[lane] = F.h[lane];
+            if (lane == 0) {
+                Q.hx = Hx;
+                Q.hy = Hy;
+                Q.cx = cx;
+                Q.cy = cy;
+                Q.id = id;
+                Q.n = left;
+            }
+        }
+        if (lane == 0) Q.ok = ok ? 1 : narrow ? 2 : 0;
+        __syncwarp();
+    }
+}
+
+// Supergroups' records for the walk of a point-mass tree (null: not worth it).
+static const SuperRec* launch_super(WalkParams<float>& P, const SpeciesTree& st, char* base, const Layout& L,
+                                    uint32_t* counter, int64_t nb, int dtype, int num_sms, cudaStream_t s)
+{
+    constexpr size_t smem = kWalkWarps * sizeof(WalkShared<LENS_POINT, float, 0, 2>);
+    static const int bps = [] {
+        if (smem > 48 * 1024)
+            cudaFuncSetAttribute(k_super, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int nb = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_super, kWalkWarps * 32, smem);
+        return std::min(std::max(nb, 1), 16);
+    }();
+    SuperRec* rec = (SuperRec*)(base + L.super);
+    P.sdelta = (const float4*)(base + L.sdelta);
+    P.counter = counter;
+    const int64_t ns = (P.n_groups + kSuperGroups - 1) / kSuperGroups;
+    const int64_t blocks = std::min<int64_t>((ns + kWalkWarps - 1) / kWalkWarps, (int64_t)num_sms * bps);
+    const void* box = base + L.bbox;  // of a single batch: ordered uint32 or FP64 images (enqueue_groups)
+    k_super<<<(unsigned)blocks, kWalkWarps * 32, smem, s>>>(P, st.node_rcm, nb == 1 && dtype != LENS_F32 ? (const unsigned long long*)box : nullptr,
+                                                            nb == 1 && dtype == LENS_F32 ? (const uint32_t*)box : nullptr, rec, (float4*)(base + L.sdelta));
+    note_launch();
+    return rec;
 }
 
 // The slices of a split direct sum, added per ray in slice order with
@@ -472,21 +887,21 @@ static int split_slices(const lens_tree* t, int64_t ng, int64_t n_rays, int64_t 
 
 // ------------------------------------------------------------- host side
 
-template <int KIND, typename T, int R, bool AO, bool DIRECT, int TILE>
+template <int KIND, typename T, int R, bool AO, bool DIRECT, int TILE, bool LOC>
 static int walk_blocks_per_sm()
 {
     static int cached = -1;
     if (cached < 0) {
         size_t smem = kWalkWarps * sizeof(WalkShared<KIND, T, TILE, tot_rays<R>()>);
         if (smem > 48 * 1024)
-            cudaFuncSetAttribute(walk_kernel<KIND, T, R, AO, DIRECT, TILE>,
+            cudaFuncSetAttribute(walk_kernel<KIND, T, R, AO, DIRECT, TILE, LOC>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         // the walk keeps its working set in shared memory and registers:
         // prefer the largest shared-memory carveout
-        cudaFuncSetAttribute(walk_kernel<KIND, T, R, AO, DIRECT, TILE>,
+        cudaFuncSetAttribute(walk_kernel<KIND, T, R, AO, DIRECT, TILE, LOC>,
                              cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         int nb = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, walk_kernel<KIND, T, R, AO, DIRECT, TILE>,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, walk_kernel<KIND, T, R, AO, DIRECT, TILE, LOC>,
                                                       kWalkWarps * 32, smem);
         cached = nb > 0 ? nb : 1;
     }
@@ -517,59 +932,102 @@ lens_status reserve_rays(lens_tree* t, int64_t n, int64_t nb, cudaStream_t s)
     return LENS_OK;
 }
 
-template <int KIND, typename T, int R, bool AO, bool DIRECT, int TILE>
+template <int KIND, typename T, int R, bool AO, bool DIRECT, int TILE, bool LOC>
 static void launch_one(const WalkParams<T>& P, int num_sms, cudaStream_t s)
 {
     size_t smem = kWalkWarps * sizeof(WalkShared<KIND, T, TILE, tot_rays<R>()>);
-    int bps = walk_blocks_per_sm<KIND, T, R, AO, DIRECT, TILE>();
-    if (bps > 16) bps = 16;  // stack slots are allocated for 16 blocks per SM
+    int bps = walk_blocks_per_sm<KIND, T, R, AO, DIRECT, TILE, LOC>();
+    // stack slots are allocated for 16 blocks per SM, a tree walk's cut slots for kCutBlocks
+    if (bps > (DIRECT ? 16 : kCutBlocks)) bps = DIRECT ? 16 : kCutBlocks;
     int grid = num_sms * bps;
-    { walk_kernel<KIND, T, R, AO, DIRECT, TILE><<<grid, kWalkWarps * 32, smem, s>>>(P); note_launch(); }
+    { walk_kernel<KIND, T, R, AO, DIRECT, TILE, LOC><<<grid, kWalkWarps * 32, smem, s>>>(P); note_launch(); }
 }
 
-template <typename T, int R, bool AO, bool DIRECT, int TILE>
+template <typename T, int R, bool AO>
 static void launch_kind(int kind, const WalkParams<T>& P, int num_sms, cudaStream_t s)
 {
-    if (kind == LENS_POINT) launch_one<LENS_POINT, T, R, AO, DIRECT, TILE>(P, num_sms, s);
-    else if (kind == LENS_GAUSS) launch_one<LENS_GAUSS, T, R, AO, DIRECT, TILE>(P, num_sms, s);
-    else launch_one<LENS_NFW, T, R, AO, DIRECT, TILE>(P, num_sms, s);
+    if (kind == LENS_POINT) launch_one<LENS_POINT, T, R, AO, true, 0, false>(P, num_sms, s);
+    else if (kind == LENS_GAUSS) launch_one<LENS_GAUSS, T, R, AO, true, 0, false>(P, num_sms, s);
+    else launch_one<LENS_NFW, T, R, AO, true, 0, false>(P, num_sms, s);
 }
 
-// tile: the near-field tile size of the tree walk (WalkBuf); the larger tile
-// is built for FP32 tree walks only (the direct sum and the FP64 tree keep
-// the standard one).
 template <typename T, int R>
-static void launch_dispatch(int kind, bool ao, bool direct, const WalkParams<T>& P, int num_sms,
-                            cudaStream_t s, int tile = 0)
+static void launch_direct(int kind, bool ao, const WalkParams<T>& P, int num_sms, cudaStream_t s)
 {
-    if (direct) {
-        if (ao) launch_kind<T, R, true, true, 0>(kind, P, num_sms, s);
-        else launch_kind<T, R, false, true, 0>(kind, P, num_sms, s);
-    } else {
-        if constexpr (sizeof(T) == 4) {
-            if (tile == 1) {
-                if (ao) launch_kind<T, R, true, false, 1>(kind, P, num_sms, s);
-                else launch_kind<T, R, false, false, 1>(kind, P, num_sms, s);
+    if (ao) launch_kind<T, R, true>(kind, P, num_sms, s);
+    else launch_kind<T, R, false>(kind, P, num_sms, s);
+}
+
+// The one-warp tree walk of all groups: in rounds of cut groups, or, from
+// kPlainGroups groups on and without expansions, the stretched groups so and
+// the others by the plain kernel (the cut form's registers cost it 5 %).
+template <int KIND, typename T, int R, bool AO, int TILE>
+static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, const Layout& L, cudaStream_t s)
+{
+    constexpr bool kF32 = sizeof(T) == 4;
+    const int sms = t->num_sms;
+    uint32_t* counter = P.counter;
+    auto cut = [&](const WalkParams<T>& Q) {
+        if constexpr (KIND == LENS_POINT && kF32) {
+            if (Q.super) {
+                launch_one<KIND, T, R, AO, false, TILE, true>(Q, sms, s);
                 return;
             }
         }
-        if (ao) launch_kind<T, R, true, false, 0>(kind, P, num_sms, s);
-        else launch_kind<T, R, false, false, 0>(kind, P, num_sms, s);
+        launch_one<KIND, T, R, AO, false, TILE, KIND == LENS_NFW && kF32>(Q, sms, s);
+    };
+    if (KIND == LENS_POINT && kF32 && !P.super && P.n_part < 8192) {
+        // (no group can reach the limit of a cut: cells and particles together
+        // are fewer than twice the particles)
+        launch_plain<KIND, T, R, AO, TILE>(P, sms, s);
+        return;
     }
+    if (P.n_groups < kPlainGroups || P.super || (KIND == LENS_NFW && kF32)) {
+        walk_rounds<T, R>(P, P.n_groups, nq, base, L, counter, cut, s, KIND == LENS_POINT && kF32);
+        return;
+    }
+    if (P.n_part > 4 * P.n_groups) {
+        // (fewer particles: even a group that meets all of them is done before
+        // the others; lens fit, 1e5 particles, 31,250 groups)
+        const uint32_t* sub = (const uint32_t*)(base + L.sub);
+        WalkParams<T> Q = P;
+        Q.sub = sub + 16;
+        Q.sub_n = sub;
+        walk_rounds<T, R>(Q, P.n_groups, nq, base, L, counter, cut, s);
+        P.gflag = (const uint8_t*)(base + L.gflag);
+        P.skip = 1;
+        cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
+        P.counter = counter;
+    }
+    launch_plain<KIND, T, R, AO, TILE>(P, sms, s);
 }
 
-// 128-ray groups (four rays per lane): the one-warp tree walk of an FP32 tree.
-template <typename T>
-static void launch_tree4(int kind, bool ao, const WalkParams<T>& P, int num_sms, cudaStream_t s, int tile)
+template <typename T, int R>
+static void walk_tree(int kind, bool ao, const WalkParams<T>& P, lens_tree* t, int nq, char* base, const Layout& L,
+                      cudaStream_t s)
 {
-    if constexpr (sizeof(T) == 4) {
-        if (tile == 1) {
-            if (ao) launch_kind<T, 4, true, false, 1>(kind, P, num_sms, s);
-            else launch_kind<T, 4, false, false, 1>(kind, P, num_sms, s);
+    auto go = [&](auto tile) {
+        constexpr int TILE = decltype(tile)::value;
+        if (kind == LENS_POINT) {
+            if (ao) walk_tree_kind<LENS_POINT, T, R, true, TILE>(P, t, nq, base, L, s);
+            else walk_tree_kind<LENS_POINT, T, R, false, TILE>(P, t, nq, base, L, s);
+        } else if (kind == LENS_GAUSS) {
+            if (ao) walk_tree_kind<LENS_GAUSS, T, R, true, TILE>(P, t, nq, base, L, s);
+            else walk_tree_kind<LENS_GAUSS, T, R, false, TILE>(P, t, nq, base, L, s);
         } else {
-            if (ao) launch_kind<T, 4, true, false, 0>(kind, P, num_sms, s);
-            else launch_kind<T, 4, false, false, 0>(kind, P, num_sms, s);
+            if (ao) walk_tree_kind<LENS_NFW, T, R, true, TILE>(P, t, nq, base, L, s);
+            else walk_tree_kind<LENS_NFW, T, R, false, TILE>(P, t, nq, base, L, s);
         }
+    };
+    // (the larger near-field tile is built for FP32 trees, 128-ray groups
+    // likewise)
+    if constexpr (sizeof(T) == 8 && R == 4) {
+        return;
+    } else if constexpr (sizeof(T) == 4) {
+        if (t->tile == 1) go(std::integral_constant<int, 1>{});
+        else go(std::integral_constant<int, 0>{});
+    } else {
+        go(std::integral_constant<int, 0>{});
     }
 }
 
@@ -638,6 +1096,9 @@ lens_status enqueue_groups(lens_tree* t, const ShootPlan& plan, const void* dx, 
     T2* gH = (T2*)(base + L.gH);
     T4* gbox = (T4*)(base + L.gbox);
     uint2* grange = (uint2*)(base + L.grange);
+    uint8_t* gflag = (uint8_t*)(base + L.gflag);
+    uint32_t* sub = (uint32_t*)(base + L.sub);
+    LENS_CUDA(cudaMemsetAsync(sub, 0, sizeof(uint32_t), s));
     if (nb == 1 && dtype == LENS_F32) {
         const int TB = 256;
         const float* fx = (const float*)dx;
@@ -656,23 +1117,26 @@ lens_status enqueue_groups(lens_tree* t, const ShootPlan& plan, const void* dx, 
         unsigned gg = grid_for((int64_t)ng * 32, TB);
         if (plan.ox == 0.0 && plan.oy == 0.0) {
             if (R == 1)
-                { k_groups32<T, 1><<<gg, TB, 0, s>>>((int64_t)ng, n, fx, fy, sv, gH, gbox, grange, ray_l, ray_idx);
+                { k_groups32<T, 1><<<gg, TB, 0, s>>>((int64_t)ng, n, fx, fy, sv, gH, gbox, grange, ray_l, ray_idx, bb,
+                                                gflag, sub);
                   note_launch(); }
             else if (R == 2)
-                { k_groups32<T, 2><<<gg, TB, 0, s>>>((int64_t)ng, n, fx, fy, sv, gH, gbox, grange, ray_l, ray_idx);
+                { k_groups32<T, 2><<<gg, TB, 0, s>>>((int64_t)ng, n, fx, fy, sv, gH, gbox, grange, ray_l, ray_idx, bb,
+                                                gflag, sub);
                   note_launch(); }
             else
-                { k_groups32<T, 4><<<gg, TB, 0, s>>>((int64_t)ng, n, fx, fy, sv, gH, gbox, grange, ray_l, ray_idx);
+                { k_groups32<T, 4><<<gg, TB, 0, s>>>((int64_t)ng, n, fx, fy, sv, gH, gbox, grange, ray_l, ray_idx, bb,
+                                                gflag, sub);
                   note_launch(); }
         } else if (R == 1) {
             { k_groups<T, 1><<<gg, TB, 0, s>>>((int64_t)ng, d_boff, d_gfirst, (int)nb, d_borig, dx, dy, dtype,
-                                             sv, gH, gbox, grange, ray_l, ray_idx); note_launch(); }
+                                             sv, gH, gbox, grange, ray_l, ray_idx, nullptr, bb, gflag, sub); note_launch(); }
         } else if (R == 2) {
             { k_groups<T, 2><<<gg, TB, 0, s>>>((int64_t)ng, d_boff, d_gfirst, (int)nb, d_borig, dx, dy, dtype,
-                                             sv, gH, gbox, grange, ray_l, ray_idx); note_launch(); }
+                                             sv, gH, gbox, grange, ray_l, ray_idx, nullptr, bb, gflag, sub); note_launch(); }
         } else {
             { k_groups<T, 4><<<gg, TB, 0, s>>>((int64_t)ng, d_boff, d_gfirst, (int)nb, d_borig, dx, dy, dtype,
-                                             sv, gH, gbox, grange, ray_l, ray_idx); note_launch(); }
+                                             sv, gH, gbox, grange, ray_l, ray_idx, nullptr, bb, gflag, sub); note_launch(); }
         }
     } else {
         const int TB = 256;
@@ -692,13 +1156,13 @@ lens_status enqueue_groups(lens_tree* t, const ShootPlan& plan, const void* dx, 
         unsigned gg = grid_for((int64_t)ng * 32, TB);
         if (R == 1)
             { k_groups<T, 1><<<gg, TB, 0, s>>>((int64_t)ng, d_boff, d_gfirst, (int)nb, d_borig, dx, dy, dtype,
-                                             sv, gH, gbox, grange, ray_l, ray_idx); note_launch(); }
+                                             sv, gH, gbox, grange, ray_l, ray_idx, d_bbox, nullptr, gflag, sub); note_launch(); }
         else if (R == 2)
             { k_groups<T, 2><<<gg, TB, 0, s>>>((int64_t)ng, d_boff, d_gfirst, (int)nb, d_borig, dx, dy, dtype,
-                                             sv, gH, gbox, grange, ray_l, ray_idx); note_launch(); }
+                                             sv, gH, gbox, grange, ray_l, ray_idx, d_bbox, nullptr, gflag, sub); note_launch(); }
         else
             { k_groups<T, 4><<<gg, TB, 0, s>>>((int64_t)ng, d_boff, d_gfirst, (int)nb, d_borig, dx, dy, dtype,
-                                             sv, gH, gbox, grange, ray_l, ray_idx); note_launch(); }
+                                             sv, gH, gbox, grange, ray_l, ray_idx, d_bbox, nullptr, gflag, sub); note_launch(); }
     }
 
     if (nb == 1) {
@@ -803,8 +1267,8 @@ static lens_status enqueue_typed(lens_tree* t, const ShootPlan& plan, const void
         P.halos = t->halos;
         P.n_halos = first_launch ? (int)t->n_halos : 0;
         P.accumulate = first_launch ? ((flags & LENS_ACCUMULATE) ? 1 : 0) : 1;
-        P.counter = counter + 2 * launches;
-        LENS_CUDA(cudaMemsetAsync(P.counter, 0, sizeof(uint32_t), s));
+        P.counter = counter + 8 * launches;
+        LENS_CUDA(cudaMemsetAsync(P.counter, 0, 8 * sizeof(uint32_t), s));
         // few ray groups in a direct sum: split the particles over slices too
         P.n_slices = direct ? split_slices(t, (int64_t)ng, n, st.n) : 1;
         P.split_n = n;
@@ -817,11 +1281,23 @@ static lens_status enqueue_typed(lens_tree* t, const ShootPlan& plan, const void
                     done = R == 1 ? launch_ws<T, 1>(st.kind, ao, P, t->num_sms, s, consumers)
                                   : launch_ws<T, 2>(st.kind, ao, P, t->num_sms, s, consumers);
             }
-            if (!done) {
-                if (R == 1) launch_dispatch<T, 1>(st.kind, ao, direct, P, t->num_sms, s, t->tile);
-                else if (R == 2) launch_dispatch<T, 2>(st.kind, ao, direct, P, t->num_sms, s, t->tile);
-                else if (!direct) launch_tree4<T>(st.kind, ao, P, t->num_sms, s, t->tile);
+            if (!done && direct) {
+                if (R == 1) launch_direct<T, 1>(st.kind, ao, P, t->num_sms, s);
+                else if (R == 2) launch_direct<T, 2>(st.kind, ao, P, t->num_sms, s);
                 else return lens_set_error(LENS_ERR_INTERNAL, "128-ray groups in a direct sum");
+            } else if (!done) {
+                const int nq = ao ? 2 : 5;
+                // supergroups from 16,384 groups (512 warps of k_super), where
+                // the caller keeps no lists and counts nothing
+                if constexpr (sizeof(T) == 4) {
+                    P.super = nullptr;
+                    if (st.kind == LENS_POINT && ng >= 16384 && !keep && !P.stats)
+                        P.super = launch_super(P, st, base, L, counter + 8 * launches + 3, nb, dtype, t->num_sms, s);
+                }
+                P.counter = counter + 8 * launches;
+                if (R == 1) walk_tree<T, 1>(st.kind, ao, P, t, nq, base, L, s);
+                else if (R == 2) walk_tree<T, 2>(st.kind, ao, P, t, nq, base, L, s);
+                else walk_tree<T, 4>(st.kind, ao, P, t, nq, base, L, s);
             }
             if (P.n_slices > 1) {
                 k_split_sum<T><<<grid_for(n, 256), 256, 0, s>>>(n, P.n_slices, ao ? 2 : 5, P.split, P.out[0], P.out[1],
@@ -840,8 +1316,8 @@ static lens_status enqueue_typed(lens_tree* t, const ShootPlan& plan, const void
         P.accumulate = (flags & LENS_ACCUMULATE) ? 1 : 0;
         P.counter = counter;
         LENS_CUDA(cudaMemsetAsync(P.counter, 0, sizeof(uint32_t), s));
-        if (R == 1) launch_dispatch<T, 1>(LENS_POINT, ao, true, P, t->num_sms, s);
-        else if (R == 2) launch_dispatch<T, 2>(LENS_POINT, ao, true, P, t->num_sms, s);
+        if (R == 1) launch_direct<T, 1>(LENS_POINT, ao, P, t->num_sms, s);
+        else if (R == 2) launch_direct<T, 2>(LENS_POINT, ao, P, t->num_sms, s);
         else return lens_set_error(LENS_ERR_INTERNAL, "128-ray groups without particles");
     }
     if (timing) {
@@ -1176,7 +1652,7 @@ static lens_status noalloc_typed(lens_tree* t, double ox, double oy, const void*
         P.n_halos = first_launch ? (int)t->n_halos : 0;
         P.accumulate = first_launch ? ((flags & LENS_ACCUMULATE) ? 1 : 0) : 1;
         P.counter = counters + launches;
-        launch_dispatch<T, 1>(sp.kind, ao, true, P, t->num_sms, s);
+        launch_direct<T, 1>(sp.kind, ao, P, t->num_sms, s);
         first_launch = false;
         ++launches;
     }
@@ -1186,7 +1662,7 @@ static lens_status noalloc_typed(lens_tree* t, double ox, double oy, const void*
         P.n_halos = (int)t->n_halos;
         P.accumulate = (flags & LENS_ACCUMULATE) ? 1 : 0;
         P.counter = counters;
-        launch_dispatch<T, 1>(LENS_POINT, ao, true, P, t->num_sms, s);
+        launch_direct<T, 1>(LENS_POINT, ao, P, t->num_sms, s);
     }
     LENS_CUDA(cudaGetLastError());
     return LENS_OK;

@@ -6,12 +6,92 @@
 // full buffer or hands it to another warp.
 #pragma once
 
+#include "local.cuh"
 #include "profiles.cuh"
 #include "walk_shared.cuh"
 
 namespace lens {
 
-template <typename T> struct WalkParams {
+// A group's walk can be cut: the warp that walks it hands the boxes still on
+// its stack (and, deferred, big lists) to `parts` work items of the next
+// launch, each of which walks every parts-th box of them for the same rays.
+// A warp's walk is a serial chain of dependent steps, so a launch of few
+// groups leaves most of the chip idle (295 groups of a 97^2-ray map: 2.9 ms
+// for 295 warps of 3,648), and a group over a density cusp runs alone at the
+// end of a launch of many (walk_rounds says when groups are cut).  Every item
+// writes its rays' totals to a slot; k_cut_sum adds the slots of a group in
+// order.  Where a cut finds its pool full, the warp itself walks the parts one
+// after another and adds their totals in the same order: the bits do not
+// depend on which warp ran what.
+constexpr int kCutNodes = 384;   // boxes handed over per cut
+constexpr int kCutRanges = 96;   // deferred big lists per cut
+constexpr int kLongList = 8;     // chunks of a big list that is deferred wherever a group may be cut
+constexpr uint32_t kNoItem = 0xffffffffu, kNoCut = 0xffffffffu;
+
+struct alignas(16) CutSlot {
+    uint32_t g;        // group
+    uint32_t base;     // its totals: slot base (before the cut), base + 1 + j (part j)
+    uint32_t parts;    // 0: not cut after all
+    uint32_t n_nodes, n_ranges;
+    int32_t parent;    // the totals go to this slot of the pool before, or -1: the outputs
+    uint32_t pad[2];
+    int2 ranges[kCutRanges];  // big lists {first entry, entries}
+    int nodes[kCutNodes];
+};
+
+static_assert(sizeof(CutSlot) == kCutSlotBytes, "scratch layout");
+
+// The cuts of one launch: cnt[0] counts cuts, cnt[1] item slots.  Every slot
+// below min(cnt[1], cap) is written by the cut that took it: item[base] =
+// kNoItem, item[base + 1 + j] = cut << 7 | j.
+template <typename T> struct CutPool {
+    uint32_t* cnt = nullptr;
+    CutSlot* slots = nullptr;
+    uint32_t max_cuts = 0, cap = 0;
+    uint32_t* item = nullptr;
+    T* part = nullptr;      // cap x 5 x 32R totals
+};
+
+template <typename T> struct CutParams {
+    CutPool<T> in;          // the items of this launch (null: whole groups)
+    CutPool<T> out;         // where this launch's cuts go (null: no cuts)
+    uint32_t limit = 0;     // evaluated entries before a group is cut
+    uint32_t limit_stretched = 0;  // the same for a stretched group (0: as the others)
+    uint32_t parts = 0;
+    int min_nodes = 0;      // boxes on the stack to be worth a cut
+    int defer = 0;          // every big list met before the cut goes to the parts
+    unsigned char* local = nullptr;  // per warp: deferred lists, and a cut's slot and sums if its pool is full
+};
+
+template <int R, typename T> constexpr size_t cut_local_bytes() { return kCutSlotBytes + 2 * 5 * 32 * R * sizeof(T); }
+
+// A supergroup: kSuperGroups consecutive groups whose common part of the walk
+// is done once (k_super).  Boxes that every group accepts, and leaves that
+// every group opens, and that lie far from the supergroup seen from its size,
+// are in its expansion h (local.cuh) about (cx, cy) in the frame anchored at
+// (hx, hy), scale 1/id; the boxes that are left are where each group's own
+// walk starts.  sdelta[g] corrects the expansion's alpha and gamma for group
+// g: at the centre of the group's box, the sum of the same sources one by one,
+// in the order and with the compensated partial sums of a group's own walk,
+// minus the expansion's value.  Over a patch much smaller than the distances
+// every ray of a group shares the rounding of that sum, and the results keep
+// it (a component that happens to be 1e-3 of the sum of |terms| otherwise
+// moves by 2e-5).
+struct SuperRec {
+    int ok;        // 1: use it; 0: each group starts at the root; 2: and takes no expansions of its own
+    int n;         // boxes left
+    float hx, hy, cx, cy, id, pad;
+    float h[kLocH];
+    int nodes[kCutNodes];
+};
+static_assert(sizeof(SuperRec) == kSuperBytes, "scratch layout");
+
+// A species' constants in the evaluation.
+template <typename T> struct EvalConsts {
+    T Uq, invNq, Uq2, Nq, eU;
+};
+
+template <typename T> struct WalkParams : EvalConsts<T> {
     const vec4_t<T>* nodeA;
     const v2_t<T>* nodeB;
     const int4* link;
@@ -22,7 +102,6 @@ template <typename T> struct WalkParams {
     const vec4_t<T>* big_chunk;  // support bounding box per 32 entries
     const vec4_t<T>* node_bigbox;
     int64_t n_part;
-    T Uq, invNq, Uq2, Nq, eU;
     const v2_t<T>* gH;
     const vec4_t<T>* gbox;
     const uint2* grange;
@@ -53,10 +132,20 @@ template <typename T> struct WalkParams {
     uint32_t* list_ids;
     uint32_t* list_n;
     int list_K;
+    CutParams<T> cut;  // parts of groups whose walk is shared by several warps
+    const uint8_t* gflag;     // per group: 1 if stretched (walk_shared.cuh)
+    // only the groups sub[0 .. *sub_n) (null: all), or all but the stretched ones
+    const uint32_t* sub;
+    const uint32_t* sub_n;
+    int skip;
+    const SuperRec* super;   // supergroups' records (null: every group starts at the root)
+    const float4* sdelta;    // per group: see SuperRec
 };
 
 // Record one traversal step's boxes that matter to the adjoint (one entry
-// per box, lane order) into the context's list, if it keeps one.
+// per box, lane order) into the context's list, if it keeps one.  The parts of
+// a cut group share the group's count in memory (rec_shared); an overflow
+// leaves it above the room.
 template <class Ctx>
 LENS_DEV void record_step(Ctx& C, int v, bool acc, bool leaf, bool big)
 {
@@ -64,6 +153,13 @@ LENS_DEV void record_step(Ctx& C, int v, bool acc, bool leaf, bool big)
     const int lane = threadIdx.x & 31;
     const uint32_t tag = (acc ? kListFar : 0u) | (leaf ? kListLeaf : 0u) | (big ? kListBig : 0u);
     const unsigned m = __ballot_sync(0xffffffffu, tag != 0u);
+    if (m == 0u) return;
+    if (C.rec_shared) {
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(C.rec_shared, (uint32_t)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        C.rec_n = (int)min(at, (uint32_t)C.rec_cap);
+    }
     const int pos = C.rec_n + __popc(m & ((1u << lane) - 1u));
     if (tag != 0u && pos < C.rec_cap) C.rec[pos] = (uint32_t)v | tag;
     C.rec_n += __popc(m);
@@ -93,6 +189,30 @@ template <int KIND, typename T, int TILE = 0> struct WalkBuf {
     float bnx[kB], bny[kB], bcl[kB], bm[kB], bme[kB], bk[kB], bw[kB], bic[kB];
 };
 
+// The work item a warp walks (a whole group, or a part of a cut one) and its
+// cut.  Warp-uniform and touched once per item or cut, so it lives in shared
+// memory: in registers it pushed the walk's hot loops into spills (headline
+// walk 22.6 -> 24.6 ms).
+struct WalkCut {
+    // the item
+    uint32_t g;          // group
+    uint32_t item;       // the part's slot of the in pool (kNoItem: a whole group)
+    int sp;              // boxes on the stack
+    const CutSlot* cs;   // the cut it is a part of, or null
+    int j, parts;        // part j of parts
+    int rn;              // deferred big lists to scan (every parts-th chunk from j), at rs
+    const int2* rs;
+    // its cut
+    uint32_t limit;      // evaluated entries before the cut (kNoCut: none)
+    int min_nodes;
+    int n_ranges;        // big lists deferred so far (in the warp's own slot)
+    uint32_t chunks;     // their chunks
+    int fired;           // was cut
+    int local;           // the parts are walked here (the pool was full)
+    uint32_t base;       // the cut's first item slot
+    int seg;             // local: the part being walked
+};
+
 // The list ranges of one traversal step (one per lane) and the Neumaier-
 // compensated totals of each lane's rays ([component][ray][lane]; touched once
 // per buffer flush, so they live here rather than in registers).
@@ -107,8 +227,39 @@ template <typename T, int NR = 2> struct WalkTot {
     T tot_s[5][NR][32], tot_c[5][NR][32];
 };
 
+// The local expansion of the group (FP32 trees) and the entries of a flush
+// that are evaluated ray by ray.
+struct WalkLocal {
+    LocalSum sum;
+    float rho2;                // sources with (d/|w0|)^2 up to this are expanded
+    uint8_t idx[2 * kBigCap];  // (buffers hold at most 256 entries)
+};
+struct NoLocal {};
+template <typename T> struct LocalBuf;
+template <> struct LocalBuf<float> { using type = WalkLocal; };
+template <> struct LocalBuf<double> { using type = NoLocal; };
+
+// What a flush needs beside its buffer: the species' constants, the group's
+// anchor and box, and every lane's rays.
+template <typename T, int NR> struct WalkRays {
+    EvalConsts<T> K;
+    v2_t<T> H;
+    vec4_t<T> box;
+    T lx[NR][32], ly[NR][32];
+};
+
 // Shared memory of one warp of the walk kernel.
 template <int KIND, typename T, int TILE = 0, int NR = 2> struct WalkShared {
+    WalkBuf<KIND, T, TILE> buf;
+    WalkRanges rng;
+    WalkTot<T, NR> tot;
+    WalkCut cut;
+    WalkRays<T, NR> ray;
+    typename LocalBuf<T>::type loc;
+};
+
+// Shared memory of one warp of the plain walk kernel.
+template <int KIND, typename T, int TILE = 0, int NR = 2> struct PlainShared {
     WalkBuf<KIND, T, TILE> buf;
     WalkRanges rng;
     WalkTot<T, NR> tot;
@@ -122,7 +273,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
     static constexpr int kQ = AO ? 2 : 5;  // components accumulated
     static constexpr int kNR = tot_rays<R>();
     using Buf = WalkBuf<KIND, T, TILE>;
-    const WalkParams<T>& P;
+    const EvalConsts<T>& K;  // the species' constants
     Buf* B;                // the buffers being evaluated
     WalkTot<T, kNR>* Tt;   // compensated totals of the lane's rays
     T lx[R], ly[R];
@@ -130,7 +281,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
     v2_t<T> H;
     vec4_t<T> box;
 
-    LENS_DEV WalkEval(const WalkParams<T>& p, Buf* b, WalkTot<T, kNR>* t) : P(p), B(b), Tt(t) {}
+    LENS_DEV WalkEval(const EvalConsts<T>& k, Buf* b, WalkTot<T, kNR>* t) : K(k), B(b), Tt(t) {}
 
     LENS_DEV void tot_zero()
     {
@@ -165,9 +316,11 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
         }
     }
 
-    LENS_DEV void eval_far(int nf)
+    // (idx: only those nf entries)
+    LENS_DEV void eval_far(int nf, const uint8_t* idx = nullptr)
     {
-        for (int c = 0; c < nf; ++c) {
+        for (int i = 0; i < nf; ++i) {
+            const int c = idx ? idx[i] : i;
             T dx = B->fdx[c], dy = B->fdy[c], M = B->fM[c], qr = B->fqr[c], qi = B->fqi[c];
 #pragma unroll
             for (int r = 0; r < R; ++r) cell_terms<T, AO>(part[r], lx[r] - dx, ly[r] - dy, M, qr, qi);
@@ -176,9 +329,10 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
     }
 
     // Leaf particles: full profile unless marked as a listed (softened) point.
-    LENS_DEV void eval_near(int nn)
+    LENS_DEV void eval_near(int nn, const uint8_t* idx = nullptr)
     {
-        for (int i = 0; i < nn; ++i) {
+        for (int e = 0; e < nn; ++e) {
+            const int i = idx ? idx[e] : e;
             vec4_t<T> q = B->n0[i];
             vec4_t<T> q1;
             if constexpr (KIND == LENS_NFW) q1 = B->n1[i];
@@ -190,7 +344,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
                 if (KIND == LENS_POINT) {
                     point_terms(q.z, r2, kb, Dp);
                 } else if (KIND == LENS_GAUSS) {
-                    if (q.w > T(0)) gauss_terms(q.z, q.w, r2, P.Uq, P.invNq, kb, kap, Dp);
+                    if (q.w > T(0)) gauss_terms(q.z, q.w, r2, K.Uq, K.invNq, kb, kap, Dp);
                     else point_terms(q.z, fmax(r2, -q.w), kb, Dp);
                 } else {
                     if (q.w > T(0)) nfw_terms(q.z, q.w, q1.x, q1.y, r2, kb, kap, Dp);
@@ -213,8 +367,8 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
         for (int r = 0; r < R; ++r) {
             Acc5<float> a;
             a.zero();
-            if (w < 0.0f) gauss_correction_fast<AO>(a, lx[r] + nx, ly[r] + ny, q1, P.Uq2, P.eU);
-            else gauss_correction<AO>(a, lx[r] + nx, ly[r] + ny, q, q1, P.Uq2, P.Nq);
+            if (w < 0.0f) gauss_correction_fast<AO>(a, lx[r] + nx, ly[r] + ny, q1, K.Uq2, K.eU);
+            else gauss_correction<AO>(a, lx[r] + nx, ly[r] + ny, q, q1, K.Uq2, K.Nq);
             pa[r].na1.x -= a.a1;
             pa[r].na2.x -= a.a2;
             if (!AO) {
@@ -237,11 +391,11 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
         const float2 w = *reinterpret_cast<const float2*>(&B->bw[i]);
         const float2 ic = *reinterpret_cast<const float2*>(&B->bic[i]);
         const float2 t_c = make_float2(-cl.x, -cl.y);
-        const float2 nmass = make_float2(-(mN.x * P.Nq), -(mN.y * P.Nq));
+        const float2 nmass = make_float2(-(mN.x * K.Nq), -(mN.y * K.Nq));
         const float2 ws = make_float2(w.x < 0.0f ? INFINITY : w.x, w.y < 0.0f ? INFINITY : w.y);
 #pragma unroll
         for (int r = 0; r < R; ++r)
-            gauss_correction_soft_x2<AO>(pa[r], LX[r], LY[r], nx, ny, t_c, kz, mN, nmass, ws, ic, P.Uq2, P.eU);
+            gauss_correction_soft_x2<AO>(pa[r], LX[r], LY[r], nx, ny, t_c, kz, mN, nmass, ws, ic, K.Uq2, K.eU);
     }
 
     template <bool EDGE>
@@ -255,7 +409,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
         const float2 kz = *reinterpret_cast<const float2*>(&B->bk[i]);
 #pragma unroll
         for (int r = 0; r < R; ++r)
-            gauss_correction_x2<AO, EDGE>(pa[r], LX[r], LY[r], nx, ny, cl, mN, nmE, kz, -P.Uq2);
+            gauss_correction_x2<AO, EDGE>(pa[r], LX[r], LY[r], nx, ny, cl, mN, nmE, kz, -K.Uq2);
     }
 
     // FP32 Gaussian big buffer in packed arithmetic: the whole-group-inside
@@ -335,22 +489,22 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
                 if (q.w < T(-1.5) && p.w < T(-1.5)) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
-                        gauss_correction_inside<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q1, P.eU);
-                        gauss_correction_inside<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p1, P.eU);
+                        gauss_correction_inside<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q1, K.eU);
+                        gauss_correction_inside<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p1, K.eU);
                     }
                 } else if (q.w < T(0) && p.w < T(0)) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
-                        gauss_correction_fast<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q1, P.Uq2, P.eU);
-                        gauss_correction_fast<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p1, P.Uq2, P.eU);
+                        gauss_correction_fast<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q1, K.Uq2, K.eU);
+                        gauss_correction_fast<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p1, K.Uq2, K.eU);
                     }
                 } else {
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
-                        if (q.w < T(0)) gauss_correction_fast<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q1, P.Uq2, P.eU);
-                        else gauss_correction<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q, q1, P.Uq2, P.Nq);
-                        if (p.w < T(0)) gauss_correction_fast<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p1, P.Uq2, P.eU);
-                        else gauss_correction<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p, p1, P.Uq2, P.Nq);
+                        if (q.w < T(0)) gauss_correction_fast<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q1, K.Uq2, K.eU);
+                        else gauss_correction<AO>(part[r], lx[r] - q.x, ly[r] - q.y, q, q1, K.Uq2, K.Nq);
+                        if (p.w < T(0)) gauss_correction_fast<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p1, K.Uq2, K.eU);
+                        else gauss_correction<AO>(part[r], lx[r] - p.x, ly[r] - p.y, p, p1, K.Uq2, K.Nq);
                     }
                 }
             }
@@ -361,8 +515,8 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
             for (int r = 0; r < R; ++r) {
                 T wx = lx[r] - q.x, wy = ly[r] - q.y;
                 if constexpr (KIND == LENS_GAUSS) {
-                    if (q.w < T(0)) gauss_correction_fast<AO>(part[r], wx, wy, q1, P.Uq2, P.eU);
-                    else gauss_correction<AO>(part[r], wx, wy, q, q1, P.Uq2, P.Nq);
+                    if (q.w < T(0)) gauss_correction_fast<AO>(part[r], wx, wy, q1, K.Uq2, K.eU);
+                    else gauss_correction<AO>(part[r], wx, wy, q, q1, K.Uq2, K.Nq);
                 } else {
                     T r2 = fma(wx, wx, wy * wy);
                     T inv = r2 > T(0) ? rcp(r2) : T(0);
@@ -378,10 +532,10 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
     }
 
     // Analytic components for every ray (Sec. 3.2 analytic models, App. B).
-    LENS_DEV void halos()
+    LENS_DEV void halos(const HaloDev* halos, int n_halos)
     {
-        for (int h = 0; h < P.n_halos; ++h) {
-            const HaloDev& hd = P.halos[h];
+        for (int h = 0; h < n_halos; ++h) {
+            const HaloDev& hd = halos[h];
             T hx = (T)((double)H.x - hd.x), hy = (T)((double)H.y - hd.y);
             int kind = hd.kind;
             T m = (T)hd.m;
@@ -422,18 +576,295 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkEval {
 
 // The walk kernel's context: evaluation plus the buffer counts, where a full
 // buffer is evaluated on the spot.
-template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkCtx : WalkEval<KIND, T, R, AO, TILE> {
+// The flushes of the walk kernel: everything a full buffer's evaluation needs
+// is in shared memory, so each is one function (its code inlined at every
+// flush site overflowed the instruction cache: 6.3 of 10 stall cycles) and the
+// traversal keeps none of its registers.  LOC (FP32 tree walks): the entries
+// far from the group, seen from its size, go to the group's local expansion
+// (local.cuh), one lane per entry; the others are evaluated for every ray.
+template <int KIND, typename T, int R, bool AO, int TILE, bool LOC> struct WalkFlush {
+    using WS = WalkShared<KIND, T, TILE, tot_rays<R>()>;
+    using Eval = WalkEval<KIND, T, R, AO, TILE>;
+    using Buf = WalkBuf<KIND, T, TILE>;
+
+    // The warp's shared memory (named here, not passed: a pointer argument
+    // would be a generic one, and every access a generic load).
+    static LENS_DEV WS& mine()
+    {
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        return reinterpret_cast<WS*>(smem_raw)[threadIdx.x >> 5];
+    }
+    static LENS_DEV Eval eval(WS& S)
+    {
+        const int lane = threadIdx.x & 31;
+        Eval E(S.ray.K, &S.buf, &S.tot);
+        E.H = S.ray.H;
+        E.box = S.ray.box;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            E.lx[r] = S.ray.lx[r][lane];
+            E.ly[r] = S.ray.ly[r][lane];
+            E.part[r].zero();
+        }
+        return E;
+    }
+    // Add entry i (this lane's, if it has one) to the list of those evaluated
+    // ray by ray; n entries are in it.
+    static LENS_DEV int keep_direct(WS& S, bool direct, int i, int n)
+    {
+        const unsigned m = __ballot_sync(0xffffffffu, direct);
+        if (direct) S.loc.idx[n + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = (uint8_t)i;
+        return n + __popc(m);
+    }
+
+    // Add the lanes' shares of h to the running coefficients (one copy of the
+    // code: the exchanges of 24 values are some 150 instructions).
+    static __device__ __noinline__ void add_h24(float4 a, float4 b, float4 c, float4 e, float4 f, float4 g)
+    {
+        WS& S = mine();
+        float u[16] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, e.x, e.y, e.z, e.w};
+        float v[8] = {f.x, f.y, f.z, f.w, g.x, g.y, g.z, g.w};
+        local_add(S.loc.sum, 0, lane_totals<16>(u));
+        local_add(S.loc.sum, 1, lane_totals<8>(v));
+    }
+    static LENS_DEV void add_h(const LocalH& H)
+    {
+        const float* v = H.v;
+        add_h24(make_float4(v[0], v[1], v[2], v[3]), make_float4(v[4], v[5], v[6], v[7]),
+                make_float4(v[8], v[9], v[10], v[11]), make_float4(v[12], v[13], v[14], v[15]),
+                make_float4(v[16], v[17], v[18], v[19]), make_float4(v[20], v[21], v[22], v[23]));
+    }
+
+    static __device__ __noinline__ void far(int nf)
+    {
+        WS& S = mine();
+        __syncwarp();
+        if constexpr (LOC) {
+            const int lane = threadIdx.x & 31;
+            const float4 box = S.ray.box;
+            const float d = box_radius(box.z, box.w);
+            LocalH H;
+            H.zero();
+            int nd = 0;
+#pragma unroll 1
+            for (int b = 0; b < nf; b += 32) {
+                const int i = b + lane;
+                bool direct = i < nf;
+                if (direct) {
+                    const float wx = box.x - S.buf.fdx[i], wy = box.y - S.buf.fdy[i];
+                    const float inv = rcp(fmaf(wx, wx, wy * wy));
+                    if (d * d * inv <= S.loc.rho2) {
+                        direct = false;
+                        H.cell(wx, wy, inv, d, S.buf.fM[i], S.buf.fqr[i], S.buf.fqi[i]);
+                    }
+                }
+                nd = keep_direct(S, direct, i, nd);
+            }
+            if (nd < nf) add_h(H);
+            __syncwarp();
+            if (nd > 0) eval(S).eval_far(nd, S.loc.idx);
+        } else {
+            eval(S).eval_far(nf);
+        }
+    }
+
+    static __device__ __noinline__ void near(int nn)
+    {
+        WS& S = mine();
+        __syncwarp();
+        if constexpr (LOC) {
+            const int lane = threadIdx.x & 31;
+            const float4 box = S.ray.box;
+            const float d = box_radius(box.z, box.w);
+            LocalH H;
+            H.zero();
+            int nd = 0;
+#pragma unroll 1
+            for (int b = 0; b < nn; b += 32) {
+                const int i = b + lane;
+                bool direct = i < nn;
+                if (direct) {
+                    const float4 q = S.buf.n0[i];
+                    const float wx = box.x - q.x, wy = box.y - q.y;
+                    const float r2 = fmaf(wx, wx, wy * wy), inv = rcp(r2);
+                    // a point mass for every ray of the group: beyond the
+                    // softening radius, or outside the support
+                    bool point = true;
+                    if constexpr (KIND != LENS_POINT) {
+                        const float lo2 = kLocNear2 * r2;
+                        point = q.w <= 0.0f ? lo2 >= -q.w : KIND == LENS_GAUSS ? lo2 * q.w > S.ray.K.Uq : lo2 > q.w;
+                    }
+                    if (point && d * d * inv <= S.loc.rho2) {
+                        direct = false;
+                        H.point(wx, wy, inv, d, q.z);
+                    }
+                }
+                nd = keep_direct(S, direct, i, nd);
+            }
+            if (nd < nn) add_h(H);
+            __syncwarp();
+            if (nd > 0) eval(S).eval_near(nd, S.loc.idx);
+        } else {
+            eval(S).eval_near(nn);
+        }
+    }
+
+    // After the last flush: the group's expansion for every ray, that of its
+    // supergroup (sr, if any) with its correction, and the analytic halos.
+    static __device__ __noinline__ void finish(const HaloDev* halos, int n_halos, const SuperRec* sr, float4 delta)
+    {
+        WS& S = mine();
+        __syncwarp();
+        if constexpr (LOC) {
+            if (sr) {
+                LocalFields& F = *reinterpret_cast<LocalFields*>(S.buf.n0);  // (flushed: free)
+                const int lane = threadIdx.x & 31;
+                if (lane < kLocH) F.h[lane] = sr->h[lane];
+                __syncwarp();
+                Eval E = eval(S);
+                const float ox = (E.H.x - sr->hx) - sr->cx, oy = (E.H.y - sr->hy) - sr->cy;
+                const float id = sr->id;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    local_eval<AO>(F, (E.lx[r] + ox) * id, (E.ly[r] + oy) * id, id, E.part[r]);
+                E.fold();
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    E.part[r].a1 = delta.x;
+                    E.part[r].a2 = delta.y;
+                    E.part[r].g1 = delta.z;
+                    E.part[r].g2 = delta.w;
+                }
+                E.fold();
+                __syncwarp();
+            }
+            LocalFields& F = *reinterpret_cast<LocalFields*>(S.buf.n0);  // (flushed: free)
+            local_finish(S.loc.sum, F);
+            Eval E = eval(S);
+            const float id = 1.0f / box_radius(E.box.z, E.box.w);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                local_eval<AO>(F, (E.lx[r] - E.box.x) * id, (E.ly[r] - E.box.y) * id, id, E.part[r]);
+            E.fold();
+            __syncwarp();
+        }
+        if (n_halos > 0) eval(S).halos(halos, n_halos);
+    }
+};
+
+// The walk kernel's context: the buffers' counts, where a full buffer is
+// evaluated on the spot.
+template <int KIND, typename T, int R, bool AO, int TILE = 0, bool LOC = false> struct WalkCtx {
     using value_type = T;
     using Buf = WalkBuf<KIND, T, TILE>;
-    static constexpr int kKind = KIND;
+    using Flush = WalkFlush<KIND, T, R, AO, TILE, LOC>;
+    static constexpr int kKind = KIND, kR = R;
+    static constexpr bool kCuts = true;
     static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
+    const WalkParams<T>& P;
+    typename Flush::WS& S;
+    Buf* B;
     WalkRanges* Rg;
+    WalkCut* Cut;
+    v2_t<T> H;
+    vec4_t<T> box;
+    // boxes visited, cells accepted, leaf particles, big entries scanned, kept
+    uint32_t c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0;
     int nf = 0, nn = 0, nb = 0;  // entries in the far, near and big buffers
     uint32_t* rec = nullptr;     // the group's kept interaction list, or null
+    uint32_t* rec_shared = nullptr;  // a part's: the group's count in memory
     int rec_n = 0, rec_cap = 0;
 
-    LENS_DEV WalkCtx(const WalkParams<T>& p, WalkShared<KIND, T, TILE, tot_rays<R>()>& s)
-        : WalkEval<KIND, T, R, AO, TILE>(p, &s.buf, &s.tot), Rg(&s.rng) {}
+    LENS_DEV WalkCtx(const WalkParams<T>& p, typename Flush::WS& s)
+        : P(p), S(s), B(&s.buf), Rg(&s.rng), Cut(&s.cut) {}
+
+    // Load group g's anchor, box and rays (lanes without a ray take the centre).
+    LENS_DEV void load_group(uint32_t g)
+    {
+        const int lane = threadIdx.x & 31;
+        H = P.gH[g];
+        box = P.gbox[g];
+        const uint2 rg = P.grange[g];
+        if (lane == 0) {
+            S.ray.K.Uq = P.Uq;
+            S.ray.K.invNq = P.invNq;
+            S.ray.K.Uq2 = P.Uq2;
+            S.ray.K.Nq = P.Nq;
+            S.ray.K.eU = P.eU;
+            S.ray.H = H;
+            S.ray.box = box;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int k = r * 32 + lane;
+            v2_t<T> l;
+            l.x = box.x;
+            l.y = box.y;
+            if (k < (int)rg.y) l = P.ray_l[rg.x + k];
+            S.ray.lx[r][lane] = l.x;
+            S.ray.ly[r][lane] = l.y;
+        }
+        nf = nn = nb = 0;
+        c_vis = c_acc = c_near = c_bigs = c_bigk = 0;
+    }
+    // Zero the totals and the expansion.
+    LENS_DEV void start()
+    {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int q = 0; q < (AO ? 2 : 5); ++q) S.tot.tot_s[q][r][lane] = S.tot.tot_c[q][r][lane] = T(0);
+        if constexpr (LOC) {
+            local_zero(S.loc.sum);
+            if (lane == 0) S.loc.rho2 = P.super && P.super[Cut->g / kSuperGroups].ok == 2 ? -1.0f : kLocRho2;
+        }
+        __syncwarp();
+    }
+    LENS_DEV T total(int r, int q) const
+    {
+        const int lane = threadIdx.x & 31;
+        return S.tot.tot_s[q][r][lane] + S.tot.tot_c[q][r][lane];
+    }
+    LENS_DEV void flush_far()
+    {
+        if (nf > 0) Flush::far(nf);
+        nf = 0;
+    }
+    LENS_DEV void flush_near()
+    {
+        if (nn > 0) Flush::near(nn);
+        nn = 0;
+    }
+    LENS_DEV void flush_big()
+    {
+        if constexpr (KIND != LENS_POINT) {
+            Flush::eval(S).eval_big(nb);
+            nb = 0;
+        }
+    }
+};
+
+// The context of the plain walk kernel (no cuts, no expansions): the rays stay
+// in registers and full buffers are evaluated inline.
+template <int KIND, typename T, int R, bool AO, int TILE = 0> struct PlainCtx : WalkEval<KIND, T, R, AO, TILE> {
+    using value_type = T;
+    using Buf = WalkBuf<KIND, T, TILE>;
+    static constexpr int kKind = KIND, kR = R;
+    static constexpr bool kCuts = false;
+    static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
+    const WalkParams<T>& P;
+    WalkRanges* Rg;
+    WalkCut* Cut = nullptr;
+    // boxes visited, cells accepted, leaf particles, big entries scanned, kept
+    uint32_t c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0;
+    int nf = 0, nn = 0, nb = 0;
+    uint32_t* rec = nullptr;
+    uint32_t* rec_shared = nullptr;
+    int rec_n = 0, rec_cap = 0;
+
+    LENS_DEV PlainCtx(const WalkParams<T>& p, Buf* b, WalkTot<T, tot_rays<R>()>* t, WalkRanges* r)
+        : WalkEval<KIND, T, R, AO, TILE>(p, b, t), P(p), Rg(r) {}
     LENS_DEV void flush_far()
     {
         this->eval_far(nf);
@@ -454,8 +885,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct WalkCtx : W
 // Append, in order, the leaf particles of up to 32 index ranges (one per
 // lane) to the near buffer, flushing it whenever fewer than 32 slots remain.
 template <class Ctx, typename T = typename Ctx::value_type>
-LENS_DEV void append_ranges(Ctx& C, int cnt, int first, const vec4_t<T>* src0, const vec4_t<T>* src1,
-                            int& n_seen, int& n_kept)
+LENS_DEV void append_ranges(Ctx& C, int cnt, int first, const vec4_t<T>* src0, const vec4_t<T>* src1)
 {
     constexpr int KIND = Ctx::kKind;
     const unsigned full = 0xffffffffu;
@@ -463,7 +893,7 @@ LENS_DEV void append_ranges(Ctx& C, int cnt, int first, const vec4_t<T>* src0, c
     int tot;
     int off = warp_exclusive_scan(cnt, &tot);
     if (tot == 0) return;
-    n_seen += tot;
+    C.c_near += (uint32_t)tot;
     C.Rg->rs_off[lane] = off;
     C.Rg->rs_first[lane] = first;
     if (lane == 31) C.Rg->rs_off[32] = tot;
@@ -498,7 +928,6 @@ LENS_DEV void append_ranges(Ctx& C, int cnt, int first, const vec4_t<T>* src0, c
             if constexpr (KIND == LENS_NFW) C.B->n1[slot] = q1;
         }
         C.nn += __popc(ball);
-        n_kept += __popc(ball);
         __syncwarp();
     }
 }
@@ -511,32 +940,29 @@ template <int KIND, typename T> LENS_DEV int big_used(int nbuf)
 }
 
 // Big lists of the visited boxes (one list per lane: entries [z, z + w) of
-// the big arrays).  A list whose support box misses the group is skipped;
-// otherwise its 32-entry chunks are tested by their support boxes and the
+// the big arrays, cnt 32-entry chunks; 0: none, or its support box misses the
+// group).  The chunks are tested by their support boxes and the
 // entries of the chunks that pass are tested one by one; entries whose
 // support reaches the group's box are appended to the big buffer.
+// With a stride, only every cstep-th chunk from c0 is taken (a part's share).
 template <class Ctx, typename T = typename Ctx::value_type>
-LENS_DEV bool append_big(Ctx& C, bool has, int v, int z, int w, int& n_seen, int& n_kept)
+LENS_DEV void append_big(Ctx& C, int cnt, int z, int w, int c0 = 0, int cstep = 1)
 {
     constexpr int KIND = Ctx::kKind;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const WalkParams<T>& P = C.P;
-    int cnt = 0;
-    if (has) {
-        vec4_t<T> nb4 = P.node_bigbox[v];
-        if (box_reaches_group<T>(nb4, C.H, C.box)) cnt = ((z + w - 1) >> 5) - (z >> 5) + 1;
-    }
     int tot;
     int off = warp_exclusive_scan(cnt, &tot);
-    if (tot == 0) return false;
+    if (tot == 0) return;
+    int n_seen = 0, n_kept = 0;
     C.Rg->rs_off[lane] = off;
     C.Rg->rs_first[lane] = z;
     C.Rg->rs_end[lane] = z + w;
     if (lane == 31) C.Rg->rs_off[32] = tot;
     __syncwarp();
-    for (int base = 0; base < tot; base += 32) {
-        int i = base + lane;
+    for (int base = c0; base < tot; base += 32 * cstep) {
+        int i = base + lane * cstep;
         int cid = -1, own = 0;
         bool pass = false;
         if (i < tot) {
@@ -614,29 +1040,113 @@ LENS_DEV bool append_big(Ctx& C, bool has, int v, int z, int w, int& n_seen, int
             __syncwarp();
         }
     }
-    return cnt > 0;
+    C.c_bigs += (uint32_t)n_seen;
+    C.c_bigk += (uint32_t)n_kept;
 }
 
 
-// Walk the tree for the context's group (Sec. 3.2): up to 32 candidate boxes
-// per step, one per lane, tested against the group's bounding box; accepted
-// boxes go to the far buffer, opened leaves to the near buffer, opened
-// internal boxes push their children, and every visited box's big list is
-// scanned.  Full buffers are flushed through the context (evaluated on the
-// spot, or handed to an evaluating warp); the caller flushes what remains.
+// The warp's own cut slot (the lists deferred so far, and the boxes of a cut
+// whose pool is full) and the sums beside it.
+template <int R, typename T> LENS_DEV unsigned char* cut_own(const CutParams<T>& cp)
+{
+    const int64_t w = (int64_t)blockIdx.x * kWalkWarps + (threadIdx.x >> 5);
+    return cp.local + w * (int64_t)cut_local_bytes<R, T>();
+}
+
+// Cut the walk: the boxes at the bottom of the stack (the shallowest) and the
+// deferred lists go to a slot of the pool, or stay in the warp's own if the
+// pool is full (1 + parts item slots are taken; those below the pool's end
+// are written whatever comes of it).  Returns how many boxes stay (at the
+// bottom of the stack).
+template <int R, typename T> LENS_DEV int cut_now(const CutParams<T>& cp, WalkCut& K, int* stack, int sp)
+{
+    const unsigned full = 0xffffffffu;
+    const uint32_t lane = threadIdx.x & 31;
+    const CutPool<T>& pool = cp.out;
+    uint32_t ci = 0, base = 0;
+    if (lane == 0) ci = atomicAdd(pool.cnt, 1u);
+    ci = __shfl_sync(full, ci, 0);
+    bool pooled = ci < pool.max_cuts;
+    if (pooled) {
+        if (lane == 0) base = atomicAdd(pool.cnt + 1, cp.parts + 1);
+        base = __shfl_sync(full, base, 0);
+        pooled = base + cp.parts + 1 <= pool.cap;
+        for (uint32_t j = lane; j < cp.parts + 1; j += 32)
+            if (base + j < pool.cap) pool.item[base + j] = pooled && j > 0 ? (ci << 7 | (j - 1)) : kNoItem;
+        if (!pooled && lane == 0) pool.slots[ci].parts = 0;
+    }
+    CutSlot* own = (CutSlot*)cut_own<R>(cp);
+    CutSlot* s = pooled ? pool.slots + ci : own;
+    const int nd = sp < kCutNodes ? sp : kCutNodes;
+    if (pooled)
+        for (int i = (int)lane; i < K.n_ranges; i += 32) s->ranges[i] = own->ranges[i];
+    for (int i = (int)lane; i < nd; i += 32) s->nodes[i] = stack[i];
+    if (lane == 0) {
+        s->g = K.g;
+        s->base = base;
+        s->parts = cp.parts;
+        s->n_nodes = (uint32_t)nd;
+        s->n_ranges = (uint32_t)K.n_ranges;
+        s->parent = K.item == kNoItem ? -1 : (int32_t)K.item;
+        K.fired = 1;
+        K.local = !pooled;
+        K.base = base;
+    }
+    __syncwarp();
+    for (int i = nd; i < sp; i += 32) {
+        const int m = i + (int)lane < sp ? stack[i + lane] : 0;
+        __syncwarp();
+        if (i + (int)lane < sp) stack[i + lane - nd] = m;
+        __syncwarp();
+    }
+    return sp - nd;
+}
+
+// Walk the tree for the context's group (Sec. 3.2) from the sp boxes on the
+// stack: up to 32 candidate boxes per step, one per lane, tested against the
+// group's bounding box; accepted boxes go to the far buffer, opened leaves to
+// the near buffer, opened internal boxes push their children, and every
+// visited box's big list is scanned.  Full buffers are flushed through the
+// context (evaluated on the spot, or handed to an evaluating warp); the caller
+// flushes what remains.  Where the walk may be cut (C.Cut->limit), long big
+// lists are put aside, and once the walk has evaluated `limit` entries (or
+// has only long lists left) it is cut.  The deferred lists of the item itself
+// (C.Cut->rn) are scanned 32 to a step, in steps without boxes.
 // Returns false if the warp's stack overflowed (the error word is set).
 template <class Ctx, typename T = typename Ctx::value_type>
-LENS_DEV bool traverse(Ctx& C, int* stack, int& c_vis, int& c_acc, int& c_near, int& c_bigs, int& c_bigk)
+LENS_DEV bool traverse(Ctx& C, int* stack, int sp)
 {
     constexpr int KIND = Ctx::kKind;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const WalkParams<T>& P = C.P;
-    int sp = 1, c_dummy = 0;
-    if (lane == 0) stack[0] = 0;
-    __syncwarp();
-    while (sp > 0) {
-        int k = sp < 32 ? sp : 32;
+    uint32_t limit = Ctx::kCuts ? C.Cut->limit : kNoCut;
+    int rn = Ctx::kCuts ? C.Cut->rn : 0;
+    for (;;) {
+        bool lists = false;  // a step of deferred lists
+        if constexpr (Ctx::kCuts && KIND != LENS_POINT) {
+            lists = rn > 0;
+            if (sp == 0 && !lists && limit != kNoCut && C.Cut->n_ranges > 0) {
+                // only deferred lists are left: worth a cut (a list's chunk
+                // keeps about half of its entries), or scanned here
+                const bool cut = 16 * C.Cut->chunks >= limit + 512;
+                limit = kNoCut;
+                if (cut) {
+                    cut_now<Ctx::kR>(P.cut, *C.Cut, stack, 0);
+                } else {
+                    rn = C.Cut->n_ranges;
+                    if (lane == 0) {
+                        C.Cut->rs = ((CutSlot*)cut_own<Ctx::kR>(P.cut))->ranges;
+                        C.Cut->j = 0;
+                        C.Cut->parts = 1;
+                    }
+                    __syncwarp();
+                    lists = true;
+                }
+            }
+        }
+        if (sp == 0 && !lists) break;
+        int k = lists ? 0 : sp < 32 ? sp : 32;
         sp -= k;
         int v = lane < k ? stack[sp + lane] : -1;
         __syncwarp();
@@ -666,8 +1176,8 @@ LENS_DEV bool traverse(Ctx& C, int* stack, int& c_vis, int& c_acc, int& c_near, 
             C.B->fqi[pos] = Q.y;
         }
         C.nf += __popc(ball);
-        c_vis += k;
-        c_acc += __popc(ball);
+        C.c_vis += (uint32_t)k;
+        C.c_acc += (uint32_t)__popc(ball);
         int nc = open ? Lk.y : 0;
         int totc;
         int offc = warp_exclusive_scan(nc, &totc);
@@ -677,17 +1187,319 @@ LENS_DEV bool traverse(Ctx& C, int* stack, int& c_vis, int& c_acc, int& c_near, 
         }
         for (int c = 0; c < nc; ++c) stack[sp + offc + c] = Lk.x + c;
         sp += totc;
-        append_ranges(C, leaf ? (Lk.y & kCountMask) : 0, Lk.x, P.leaf0, P.leaf1, c_near, c_dummy);
+        append_ranges(C, leaf ? (Lk.y & kCountMask) : 0, Lk.x, P.leaf0, P.leaf1);
         bool big = false;
-        if constexpr (KIND != LENS_POINT) big = append_big(C, valid && Lk.w > 0, v, Lk.z, Lk.w, c_bigs, c_bigk);
+        if constexpr (KIND != LENS_POINT) {
+            int cnt = 0, c0 = 0, cstep = 1;
+            if (lists) {
+                const int i = rn - 1 - lane;
+                if (i >= 0) {
+                    const int2 r = C.Cut->rs[i];
+                    Lk.z = r.x;
+                    Lk.w = r.y;
+                }
+                c0 = C.Cut->j;
+                cstep = C.Cut->parts;
+                rn = rn > 32 ? rn - 32 : 0;
+            } else if (valid && Lk.w > 0) {
+                big = box_reaches_group<T>(P.node_bigbox[v], C.H, C.box);
+                if (!big) Lk.w = 0;
+            }
+            if (Lk.w > 0 && (lists || big)) cnt = ((Lk.z + Lk.w - 1) >> 5) - (Lk.z >> 5) + 1;
+            if constexpr (Ctx::kCuts) {
+                if (!lists && limit != kNoCut) {
+                    const bool put = cnt > (P.cut.defer ? 0 : kLongList);
+                    const unsigned bm = __ballot_sync(full, put);
+                    if (bm) {
+                        const int n0 = C.Cut->n_ranges, pos = n0 + __popc(bm & ((1u << lane) - 1u));
+                        uint32_t ch = 0;
+                        if (put && pos < kCutRanges) {
+                            ((CutSlot*)cut_own<Ctx::kR>(P.cut))->ranges[pos] = make_int2(Lk.z, Lk.w);
+                            ch = (uint32_t)cnt;
+                            cnt = 0;
+                        }
+                        ch = __reduce_add_sync(full, ch);
+                        if (lane == 0) {
+                            C.Cut->n_ranges = min(n0 + __popc(bm), kCutRanges);
+                            C.Cut->chunks += ch;
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+            append_big(C, cnt, Lk.z, Lk.w, c0, cstep);
+        }
         record_step(C, v, acc, leaf, big);
         __syncwarp();
         if (C.nf >= 32) {
             C.flush_far();
             __syncwarp();
         }
+        if constexpr (Ctx::kCuts) {
+            const uint32_t work = C.c_near + C.c_bigk + (C.c_acc >> 1) + (C.c_bigs >> 4);
+            if (work >= limit && sp >= C.Cut->min_nodes) {
+                sp = cut_now<Ctx::kR>(P.cut, *C.Cut, stack, sp);
+                limit = kNoCut;
+            }
+        }
     }
     return true;
+}
+
+// Put the boxes of the item's part on the stack, and its share of the lists.
+LENS_DEV void load_part(WalkCut& K, int* stack)
+{
+    const int lane = threadIdx.x & 31, nn = (int)K.cs->n_nodes, j = K.j, parts = K.parts;
+    const int sp = nn > j ? (nn - j + parts - 1) / parts : 0;
+    for (int i = lane; i < sp; i += 32) stack[i] = K.cs->nodes[j + i * parts];
+    __syncwarp();
+    if (lane == 0) {
+        K.sp = sp;
+        K.rn = (int)K.cs->n_ranges;
+        K.rs = K.cs->ranges;
+    }
+    __syncwarp();
+}
+
+// Take the next item (false: none left); its boxes go on the stack.
+template <typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int* stack, WalkCut& K)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const CutPool<T>& in = P.cut.in;
+    const int64_t n = in.cnt ? (int64_t)min(in.cnt[1], in.cap) : P.sub ? (int64_t)*P.sub_n : P.n_groups;
+    for (;;) {
+        uint32_t item = 0;
+        if (lane == 0) item = atomicAdd(P.counter, 1u);
+        item = __shfl_sync(full, item, 0);
+        if ((int64_t)item >= n) return false;
+        uint32_t e = 0;
+        if (in.cnt) {
+            e = in.item[item];
+            if (e == kNoItem) continue;
+        } else if (P.skip && P.gflag[P.order ? P.order[item] : item]) {
+            continue;
+        }
+        if (lane == 0) {
+            K.limit = P.cut.out.cnt ? P.cut.limit : kNoCut;
+            K.min_nodes = P.cut.min_nodes;
+            K.n_ranges = 0;
+            K.chunks = 0;
+            K.fired = K.local = 0;
+            K.seg = 0;
+            K.rn = 0;
+            if (in.cnt) {
+                const CutSlot* cs = in.slots + (e >> 7);
+                K.cs = cs;
+                K.j = (int)(e & 127u);
+                K.parts = (int)cs->parts;
+                K.g = cs->g;
+                K.item = item;
+            } else {
+                K.cs = nullptr;
+                K.g = P.sub ? P.sub[item] : P.order ? P.order[item] : item;
+                if (P.cut.limit_stretched && P.cut.out.cnt && P.gflag[K.g]) K.limit = P.cut.limit_stretched;
+                K.item = kNoItem;
+                K.sp = 1;
+                stack[0] = 0;
+            }
+        }
+        __syncwarp();
+        if (in.cnt) {
+            load_part(K, stack);
+        } else if (P.super) {
+            // the boxes that the supergroup's walk left
+            const SuperRec& sr = P.super[K.g / kSuperGroups];
+            if (sr.ok == 1) {
+                const int n = sr.n;
+                for (int i = lane; i < n; i += 32) stack[i] = sr.nodes[i];
+                __syncwarp();
+                if (lane == 0) K.sp = n;
+                __syncwarp();
+            }
+        }
+        return true;
+    }
+}
+
+// A cut whose pool was full: after each segment (the group's own, then each
+// part) its totals are added to the sums beside the warp's slot, as k_cut_sum
+// adds them; then the next part's boxes go on the stack.  False: no part left.
+template <int R, int NQ, typename T, class Tot>
+LENS_DEV bool local_next_part(const CutParams<T>& cp, WalkCut& K, int* stack, Tot&& tot)
+{
+    const int lane = threadIdx.x & 31, seg = K.seg;
+    unsigned char* own = cut_own<R>(cp);
+    T* sums = (T*)(own + kCutSlotBytes);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            T* a = sums + ((q * R + r) * 2) * 32 + lane;
+            T s = seg ? a[0] : tot(r, q), c = seg ? a[32] : T(0);
+            if (seg) Comp5<T>::add1(s, c, tot(r, q));
+            a[0] = s;
+            a[32] = c;
+        }
+    __syncwarp();
+    if (seg == (int)cp.parts) return false;
+    if (lane == 0) {
+        K.cs = (CutSlot*)own;
+        K.j = seg;
+        K.parts = (int)cp.parts;
+        K.seg = seg + 1;
+        K.limit = kNoCut;
+    }
+    __syncwarp();
+    load_part(K, stack);
+    return true;
+}
+template <int R, typename T> LENS_DEV T local_total(const CutParams<T>& cp, int r, int q)
+{
+    const T* a = (const T*)(cut_own<R>(cp) + kCutSlotBytes) + ((q * R + r) * 2) * 32 + (threadIdx.x & 31);
+    return a[0] + a[32];
+}
+
+// Where an item's totals go: the outputs (null), its own slot, or, when it was
+// cut, the cut's first slot.
+template <int R, typename T> LENS_DEV T* item_totals(const CutParams<T>& cp, const WalkCut& K)
+{
+    if (K.fired && !K.local) return cp.out.part + (int64_t)K.base * (5 * 32 * R);
+    if (K.item != kNoItem) return cp.in.part + (int64_t)K.item * (5 * 32 * R);
+    return nullptr;
+}
+
+// Add an item's counts to the walk counters (LENS_COUNT) and to its group's
+// work record.
+template <class Ctx> LENS_DEV void count_item(const Ctx& C, uint32_t g, uint32_t n_rays, bool head)
+{
+    const auto& P = C.P;
+    if ((threadIdx.x & 31) != 0) return;
+    if (P.gcost) atomicAdd(P.gcost + g, C.c_vis + C.c_acc + C.c_near + C.c_bigk);
+    if (P.stats) {
+        if (head) atomicAdd(&P.stats[0], 1ull);
+        atomicAdd(&P.stats[1], (unsigned long long)C.c_vis);
+        atomicAdd(&P.stats[2], (unsigned long long)C.c_acc);
+        atomicAdd(&P.stats[3], (unsigned long long)C.c_near);
+        atomicAdd(&P.stats[4], (unsigned long long)C.c_bigs);
+        atomicAdd(&P.stats[5], (unsigned long long)C.c_bigk);
+        atomicAdd(&P.stats[6], (unsigned long long)n_rays * (C.c_acc + C.c_near + C.c_bigk));
+    }
+}
+
+// The totals of every cut group of `pool`, its parts added in order with
+// Neumaier compensation, into the outputs, or into the slot of the part that
+// was cut again (`to`).  One warp per (cut, component).
+template <typename T, int R>
+__global__ void k_cut_sum(CutPool<T> pool, CutPool<T> to, WalkParams<T> P, int nq)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t nc = min(pool.cnt[0], pool.max_cuts) * (uint32_t)nq;
+    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
+    constexpr int64_t stride = 5 * 32 * R;
+    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nc; w += nw) {
+        const CutSlot& cs = pool.slots[w / (uint32_t)nq];
+        const int q = (int)(w % (uint32_t)nq), parts = (int)cs.parts;
+        if (parts == 0) continue;
+        const uint2 rg = P.grange[cs.g];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const T* p = pool.part + (int64_t)cs.base * stride + (q * R + r) * 32 + lane;
+            T s = p[0], c = T(0);
+#pragma unroll 8
+            for (int j = 1; j <= parts; ++j) Comp5<T>::add1(s, c, p[j * stride]);
+            T val = s + c;
+            if (cs.parent >= 0) {
+                to.part[(int64_t)cs.parent * stride + (q * R + r) * 32 + lane] = val;
+            } else if (r * 32 + lane < (int)rg.y && P.out[q]) {
+                const uint32_t i = P.ray_idx[rg.x + r * 32 + lane];
+                if (P.accumulate) val += P.out[q][i];
+                P.out[q][i] = val;
+            }
+        }
+    }
+}
+
+// The launches of one tree walk over ng groups: `walk(P)` launches the
+// kernel.  Groups are cut in a launch's kernel and their parts run in the
+// next one; a part may be cut once more.  Launches without items cost about
+// 3 us each, beside walks of 100 us and more.
+//   ng <= 512: far fewer warps than the chip holds.  Every group is cut as
+//     soon as its stack holds 64 boxes (its big lists deferred to the parts),
+//     into enough parts for about 8,192 warps.
+//   ng <= 4096: a group is cut after a share of work that about doubles the
+//     launch's warps.
+//   above: only a group far heavier than the others (16,384 entries and more;
+//     an average one evaluates 5,000 to 7,000), or a stretched one (which may
+//     hold most of the tree) beyond 8,192.
+//   keep_order (FP32 point masses): none but the heavy ones.  Over a patch much
+//     smaller than the distances all rays share the rounding of one sum of
+//     thousands of terms, which shows in a component that happens to be small
+//     (1e-3 of the sum of |terms|): such groups keep their order of summation.
+// Which groups are cut depends on their own walk alone.
+template <typename T, int R, typename Walk>
+void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& L, uint32_t* counter, Walk&& walk,
+                 cudaStream_t s, bool keep_order = false)
+{
+    // counter: 8 words, zeroed by the caller: work counters, then each pool's
+    CutPool<T> pool[2];
+    char *slot = base + L.cut_slot, *item = base + L.cut_item, *part = base + L.cut_part;
+    for (int k = 0; k < 2; ++k) {
+        pool[k].cnt = counter + 4 + 2 * k;
+        pool[k].slots = (CutSlot*)slot;
+        pool[k].max_cuts = kCutMax[k];
+        pool[k].item = (uint32_t*)item;
+        pool[k].part = (T*)part;
+        const size_t fit = kCutItems[k] * kCutPartBytes / (5 * 32 * R * sizeof(T));
+        pool[k].cap = (uint32_t)(fit < kCutItems[k] ? fit : kCutItems[k]);
+        slot += kCutMax[k] * kCutSlotBytes;
+        item += kCutItems[k] * sizeof(uint32_t);
+        part += kCutItems[k] * kCutPartBytes;
+    }
+    constexpr int rounds = 3;
+    CutParams<T> c[rounds];
+    P.gflag = (const uint8_t*)(base + L.gflag);
+    if (ng <= 512 && !keep_order) {
+        const int64_t want = 8192 / (ng > 0 ? ng : 1);
+        c[0].parts = (uint32_t)(want < 16 ? 16 : want > 64 ? 64 : want);
+        c[0].limit = 0;
+        c[0].min_nodes = 64;
+        c[0].defer = 1;
+        c[1].parts = 16;
+        c[1].limit = 512;
+        c[1].min_nodes = 16;
+    } else if (ng <= 4096 && !keep_order) {
+        // (every group may be cut without filling the pool: a part walked by
+        // the group's own warp is not cut again, one of the pool may be)
+        const uint32_t fit = pool[0].cap / (uint32_t)ng - 1;
+        c[0].parts = fit < 16 ? fit : 16;
+        c[0].limit = (uint32_t)(ng / 4 + 256);
+        c[0].min_nodes = 32;
+        c[1].parts = 16;
+        c[1].limit = c[0].limit;
+        c[1].min_nodes = 16;
+    } else {
+        c[0].parts = 8;
+        c[0].limit = (uint32_t)(ng <= 10922 || keep_order ? 16384 : 3 * (ng / 2));
+        c[0].limit_stretched = 8192;
+        c[0].min_nodes = 32;
+        c[1].parts = 32;
+        c[1].limit = 8192;
+        c[1].min_nodes = 16;
+    }
+    for (int r = 0; r < rounds; ++r) {
+        c[r].local = (unsigned char*)(base + L.cut_local);
+        P.counter = counter + r;
+        if (r > 0) c[r].in = pool[r - 1];
+        if (r + 1 < rounds) c[r].out = pool[r];
+        P.cut = c[r];
+        walk(P);
+    }
+    for (int r = rounds - 2; r >= 0; --r) {
+        const int64_t most = r > 0 || kCutMax[r] < ng ? kCutMax[r] : ng;
+        k_cut_sum<T, R><<<(unsigned)((most * nq + 7) / 8), 256, 0, s>>>(pool[r], r > 0 ? pool[r - 1] : CutPool<T>{}, P, nq);
+        note_launch();
+    }
 }
 
 // Launch the producer/consumer form of the walk (walk_ws.cu); false if it

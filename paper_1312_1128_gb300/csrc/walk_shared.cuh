@@ -44,14 +44,38 @@ LENS_DEV bool box_reaches_group(const vec4_t<T>& b, const v2_t<T>& H, const vec4
 
 struct Layout {
     size_t boff, borig, gfirst, bbox, k0, k1, v0, v1, tmp, rl, ridx, gH, gbox, grange, counter,
-        stack, split, gcost, heavy, total;
+        stack, split, gcost, heavy, cut_slot, cut_item, cut_part, cut_local, super, sdelta, gflag, sub, total;
 };
+
+// Cut groups (walk_dev.cuh): two pools, for the cuts of a call's first launch
+// and of its second; slots of kCutSlotBytes, item slots, and totals of
+// 5 x 32 R values per item slot.
+constexpr uint32_t kCutMax[2] = {4096, 2048}, kCutItems[2] = {32768, 16384};
+constexpr size_t kCutSlotBytes = 2336;
+// Stretched groups: Morton order jumps between quadrants, so unless the rays
+// fill power-of-two squares a few groups span half the map and open most of
+// the tree (one warp then walked on for 18 of 20 ms at 700^2 rays through 3e5
+// particles).  A group is stretched if a side of its box is over kStretch
+// times that of an even share of its batch.  From kPlainGroups groups on a
+// walk takes them in launches of their own, where they are cut early
+// (walk_dev.cuh), and the others in the plain kernel.
+constexpr int64_t kPlainGroups = 24576;
+constexpr float kStretch = 16.0f;
+
+// Supergroups (walk_dev.cuh): kSuperGroups consecutive groups, one record each.
+constexpr int kSuperGroups = 32;
+constexpr size_t kSuperBytes = 1664;
+constexpr int kCutBlocks = 8;  // resident blocks per SM of a tree walk (each warp has its own slot and sums)
+constexpr size_t kCutPartBytes = 5 * 64 * 4;  // per item slot (R = 2 in FP32); fewer item slots fit wider totals
 
 // Tags of a kept interaction-list entry (LENS_KEEP_LISTS): the box's index
 // in the low 29 bits; a box may be accepted (far cell) or an opened leaf, and
 // its big list may reach the group as well.
 constexpr uint32_t kListFar = 1u << 31, kListLeaf = 1u << 30, kListBig = 1u << 29, kListIdMask = kListBig - 1u;
-constexpr uint32_t kListOverflow = 0xffffffffu;  // list_n value of a group whose lists did not fit
+constexpr uint32_t kListOverflow = 0xffffffffu;  // list_n value of a group without lists
+// list_n of a group whose lists did not fit (parts of a cut group may still
+// add their counts to it): any value above the room says so
+constexpr uint32_t kListTooLong = 0x80000000u;
 
 // Split heavy groups (heavy_first_order): at most kHeavyGroups groups, each
 // in at most 32 slices; the plan's table holds one entry per slice.
@@ -81,11 +105,20 @@ inline Layout make_layout(int64_t n, int64_t nb, int64_t slots)
     L.gH = o; o += al(ng * 2 * sizeof(double));
     L.gbox = o; o += al(ng * 4 * sizeof(double));
     L.grange = o; o += al(ng * sizeof(uint2));
-    L.counter = o; o += al(64 * sizeof(uint32_t));
+    L.counter = o; o += al(64 * sizeof(uint32_t));  // 8 words for each species' launches
     L.stack = o; o += al((size_t)slots * kStackCap * sizeof(int));
     L.split = o; o += al(split_values(slots) * 5 * sizeof(double));
     L.gcost = o; o += al(ng * sizeof(uint32_t));
     L.heavy = o; o += al(64 + (size_t)kHeavyItems * sizeof(uint32_t));
+    L.cut_slot = o; o += al((kCutMax[0] + kCutMax[1]) * kCutSlotBytes);
+    L.cut_item = o; o += al((kCutItems[0] + kCutItems[1]) * sizeof(uint32_t));
+    L.cut_part = o; o += al((kCutItems[0] + kCutItems[1]) * kCutPartBytes);
+    // (slots = 16 blocks per SM x kWalkWarps; sums of 5 x 128 FP32 or 64 FP64 values and their corrections)
+    L.cut_local = o; o += al((size_t)slots / 16 * kCutBlocks * (kCutSlotBytes + 2 * 5 * 128 * sizeof(float)));
+    L.super = o; o += al((size_t)(ng / kSuperGroups + 1) * kSuperBytes);
+    L.sdelta = o; o += al(ng * 4 * sizeof(float));
+    L.gflag = o; o += al(ng);
+    L.sub = o; o += al((ng + 16) * sizeof(uint32_t));  // count, then (from word 16) the stretched groups
     L.total = o;
     return L;
 }

@@ -98,12 +98,16 @@ LENS_DEV bool mbar_wait(unsigned long long* b, uint32_t parity, uint32_t* err, l
 template <int KIND, typename T, int CONS> struct WsProducer {
     using value_type = T;
     using Buf = WalkBuf<KIND, T>;
-    static constexpr int kKind = KIND;
+    static constexpr int kKind = KIND, kR = 1;
+    static constexpr bool kCuts = false;  // (the team's slots go to its consumers)
     static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
     const WalkParams<T>& P;
     WsPair<KIND, T, CONS>& W;
     WalkBuf<KIND, T>* B = nullptr;
     WalkRanges* Rg;
+    WalkCut* Cut = nullptr;  // (a team's group is never cut)
+    // boxes visited, cells accepted, leaf particles, big entries scanned, kept
+    uint32_t c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0;
     v2_t<T> H;
     vec4_t<T> box;
     int nf = 0, nn = 0, nb = 0;
@@ -111,6 +115,7 @@ template <int KIND, typename T, int CONS> struct WsProducer {
     uint32_t use = 0;  // slots handed over so far
     bool alive = true;
     uint32_t* rec = nullptr;  // the group's kept interaction list, or null
+    uint32_t* rec_shared = nullptr;
     int rec_n = 0, rec_cap = 0;
 
     LENS_DEV WsProducer(const WalkParams<T>& p, WsPair<KIND, T, CONS>& w) : P(p), W(w), Rg(&w.rng) {}
@@ -174,25 +179,17 @@ LENS_DEV void ws_produce(const WalkParams<T>& P, WsPair<KIND, T, CONS>& W, int* 
         C.g = (int)g;
         C.H = P.gH[g];
         C.box = P.gbox[g];
-        int c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0;
+        if (lane == 0) stack[0] = 0;
+        __syncwarp();
+        C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
         C.rec = P.list_ids ? P.list_ids + (int64_t)g * P.list_K : nullptr;
         C.rec_n = 0;
         C.rec_cap = P.list_K;
-        const bool whole = traverse(C, stack, c_vis, c_acc, c_near, c_bigs, c_bigk);
+        const bool whole = traverse(C, stack, 1);
         C.handoff(kWsLast);
         if (!C.alive) return;
-        if (C.rec && lane == 0) P.list_n[g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListOverflow;
-        if (P.gcost && lane == 0) P.gcost[g] += (uint32_t)(c_vis + c_acc + c_near + c_bigk);
-        if (P.stats && lane == 0) {
-            unsigned long long nr = P.grange[g].y;
-            atomicAdd(&P.stats[0], 1ull);
-            atomicAdd(&P.stats[1], (unsigned long long)c_vis);
-            atomicAdd(&P.stats[2], (unsigned long long)c_acc);
-            atomicAdd(&P.stats[3], (unsigned long long)c_near);
-            atomicAdd(&P.stats[4], (unsigned long long)c_bigs);
-            atomicAdd(&P.stats[5], (unsigned long long)c_bigk);
-            atomicAdd(&P.stats[6], nr * (unsigned long long)(c_acc + c_near + c_bigk));
-        }
+        if (C.rec && lane == 0) P.list_n[g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListTooLong;
+        count_item(C, g, P.grange[g].y, true);
     }
 }
 
@@ -245,7 +242,7 @@ LENS_DEV void ws_consume(const WalkParams<T>& P, WsPair<KIND, T, CONS>& W, int c
         __syncwarp();
         mbar_arrive(&W.empty[s]);
         if (flags & kWsLast) {
-            if (P.n_halos > 0) E.halos();
+            if (P.n_halos > 0) E.halos(P.halos, P.n_halos);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (!rv[r]) continue;
