@@ -28,9 +28,8 @@
 //   A = conj(alpha)).  Since dM = dm_i, dz_cm = (dm_i d_i + m_i dz_i)/M and
 //   dQ2 = dm_i d_i^2 + 2 m_i d_i dz_i (d_i = z_i - z_cm), a particle inside
 //   the cell receives dL/dm_i = Re P(d_i) and dL/dz_i = m_i P'(d_i) with the
-//   quadratic P(d) = a + (B/M) d + C d^2.  The polynomials of all accepted
-//   ancestors are re-centred and summed from the root down, then evaluated at
-//   every particle of every leaf.
+//   quadratic P(d) = a + (B/M) d + C d^2.  Every leaf re-centres and sums the
+//   polynomials of its ancestors and evaluates them at its particles.
 #include <algorithm>
 #include <cmath>
 
@@ -79,7 +78,7 @@ template <typename T> struct BackParams {
     const uint32_t* heavy;
     // the forward's kept interaction lists (LENS_KEEP_LISTS), or null: group
     // g replays list_ids[g * list_K ...] (list_n[g] entries) instead of
-    // walking the tree, unless list_n[g] is kListOverflow
+    // walking the tree, unless list_n[g] is above list_K
     const uint32_t* list_ids;
     const uint32_t* list_n;
     int list_K;
@@ -742,65 +741,52 @@ back_kernel(BackParams<T> P)
 
 // ------------------------------------------- polynomial push-down
 
-// P_v(z) = a + b (z - z_v) + c (z - z_v)^2 (a real, b and c complex) for node v:
-// its own cell adjoint plus its parent's polynomial re-centred at v's centre
-// of mass.  One launch per level, root first.
+// Every leaf sums the polynomials of the cells it lies in, its own and its
+// ancestors', re-centred at its centre of mass z:
+//   P(d) = sum_v a_v + (B_v/M_v) (z - z_v + d) + C_v (z - z_v + d)^2
+// (a real, B and C complex: the cell adjoints dL/dM, dL/dz_cm, dL/dQ2), then
+// gives every particle dL/dm += Re P(d), dL/dz += m P'(d), and scatters (with
+// the direct terms) to the caller's input order; the size gradient is -(2/s)
+// sum kappa (G.w) with s the particle's size (r_sm from c = 1/(2 r_sm^2) of a
+// Gaussian record, r_s = 1/B of an NFW record).
+// A leaf climbs its 10 to 14 parent links itself: one launch, where pushing
+// the polynomials down level by level took one launch per level (12 of 6 us
+// at 1e5 particles) and a host wait for the level table.  adj == null (direct
+// sum): no cells.
 template <typename T>
-__global__ void k_push(uint32_t b0, uint32_t b1, const int* parent, const vec4_t<T>* nodeA, const double* adj,
-                       dbl4* polyA, double2* polyC)
-{
-    uint32_t v = b0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= b1) return;
-    vec4_t<T> A = nodeA[v];
-    const double* a = adj + 5 * (int64_t)v;
-    double M = (double)A.z;
-    double pa = a[0], pbr = 0, pbi = 0, pcr = a[1], pci = a[2];
-    if (M != 0.0) {
-        pbr = a[3] / M;
-        pbi = a[4] / M;
-    }
-    int p = parent[v];
-    if (p >= 0) {
-        dbl4 PA = polyA[p];        // {a, b_re, b_im, unused}
-        double2 PC = polyC[p];     // c
-        vec4_t<T> Ap = nodeA[p];
-        double dx = (double)A.x - (double)Ap.x, dy = (double)A.y - (double)Ap.y;  // delta = z_v - z_p
-        // a + b delta + c delta^2 (real part), b + 2 c delta, c
-        double d2x = dx * dx - dy * dy, d2y = 2.0 * dx * dy;
-        pa += PA.x + (PA.y * dx - PA.z * dy) + (PC.x * d2x - PC.y * d2y);
-        pbr += PA.y + 2.0 * (PC.x * dx - PC.y * dy);
-        pbi += PA.z + 2.0 * (PC.x * dy + PC.y * dx);
-        pcr += PC.x;
-        pci += PC.y;
-    }
-    polyA[v] = make_dbl4(pa, pbr, pbi, 0.0);
-    polyC[v] = make_double2(pcr, pci);
-}
-
-// Every particle of every leaf: dL/dm += Re P(d), dL/dz += m P'(d), then
-// scatter (with the direct terms) to the caller's input order; the size
-// gradient is -(2/s) sum kappa (G.w) with s the particle's size (r_sm from
-// c = 1/(2 r_sm^2) of a Gaussian record, r_s = 1/B of an NFW record).
-template <typename T>
-__global__ void k_leafgrad(uint32_t n_nodes, const int4* link, const vec4_t<T>* nodeA, const vec4_t<T>* exact0,
-                           const vec4_t<T>* exact1, int kind, const dbl4* polyA, const double2* polyC,
+__global__ void k_leafgrad(uint32_t n_nodes, const int4* link, const int* parent, const vec4_t<T>* nodeA,
+                           const vec4_t<T>* exact0, const vec4_t<T>* exact1, int kind, const double* adj,
                            const double* gpart, const uint32_t* perm, T* out)
 {
     uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n_nodes) return;
     int4 L = link[v];
     if (!(L.y & kLeafBit)) return;
-    vec4_t<T> A = nodeA[v];
-    dbl4 PA = polyA[v];
-    double2 PC = polyC[v];
+    const vec4_t<T> A = nodeA[v];
+    double pa = 0.0, pbr = 0.0, pbi = 0.0, pcr = 0.0, pci = 0.0;
+    if (adj) {
+        for (int u = (int)v; u >= 0; u = parent[u]) {
+            const double* a = adj + 5 * (int64_t)u;
+            const vec4_t<T> Au = nodeA[u];
+            const double M = (double)Au.z, im = M != 0.0 ? 1.0 / M : 0.0;
+            const double br = a[3] * im, bi = a[4] * im, cr = a[1], ci = a[2];
+            const double dx = (double)A.x - (double)Au.x, dy = (double)A.y - (double)Au.y;
+            const double d2x = dx * dx - dy * dy, d2y = 2.0 * dx * dy;
+            pa += a[0] + (br * dx - bi * dy) + (cr * d2x - ci * d2y);
+            pbr += br + 2.0 * (cr * dx - ci * dy);
+            pbi += bi + 2.0 * (cr * dy + ci * dx);
+            pcr += cr;
+            pci += ci;
+        }
+    }
     int cnt = L.y & kCountMask;
     for (int k = 0; k < cnt; ++k) {
         int j = L.x + k;
         vec4_t<T> q = exact0[j];
         double dx = (double)q.x - (double)A.x, dy = (double)q.y - (double)A.y;
         double d2x = dx * dx - dy * dy, d2y = 2.0 * dx * dy;
-        double gm = PA.x + (PA.y * dx - PA.z * dy) + (PC.x * d2x - PC.y * d2y);
-        double kr = PA.y + 2.0 * (PC.x * dx - PC.y * dy), ki = PA.z + 2.0 * (PC.x * dy + PC.y * dx);
+        double gm = pa + (pbr * dx - pbi * dy) + (pcr * d2x - pci * d2y);
+        double kr = pbr + 2.0 * (pcr * dx - pci * dy), ki = pbi + 2.0 * (pcr * dy + pci * dx);
         double m = (double)q.z;
         const double* gp = gpart + 4 * (int64_t)j;
         // dL = Re(m P'(d) dz): dL/dx = m Re P', dL/dy = -m Im P'
@@ -900,14 +886,10 @@ static lens_status backward_typed(lens_tree* t, double ox, double oy, const void
         if (!want && !halos_here) continue;
         double* adj = nullptr;
         double* gpart = nullptr;
-        dbl4* polyA = nullptr;
-        double2* polyC = nullptr;
         StreamTemps tmps(s);  // this species' accumulators, released on every return path
         if (st.n > 0) {
             LENS_CUDA(tmps.get(&adj, st.n_nodes * 5 * sizeof(double)));
             LENS_CUDA(tmps.get(&gpart, st.n * 4 * sizeof(double)));
-            LENS_CUDA(tmps.get(&polyA, st.n_nodes * sizeof(dbl4)));
-            LENS_CUDA(tmps.get(&polyC, st.n_nodes * sizeof(double2)));
             LENS_CUDA(cudaMemsetAsync(adj, 0, st.n_nodes * 5 * sizeof(double), s));
             LENS_CUDA(cudaMemsetAsync(gpart, 0, st.n * 4 * sizeof(double), s));
         }
@@ -939,22 +921,9 @@ static lens_status backward_typed(lens_tree* t, double ox, double oy, const void
         else back_dispatch<T, false>(kind, P, t->num_sms, s);
         if (want) {
             const int TB = 256;
-            if (!direct) {
-                LENS_TRY(finish_species(const_cast<SpeciesTree&>(st)));  // the level table
-                for (int l = 0; l <= st.depth; ++l) {
-                    uint32_t b0 = (uint32_t)st.level_start[l], b1 = (uint32_t)st.level_start[l + 1];
-                    if (b1 > b0)
-                        { k_push<T><<<grid_for(b1 - b0, TB), TB, 0, s>>>(b0, b1, st.parent, (const T4*)st.nodeA, adj,
-                                                                      polyA, polyC); note_launch(); }
-                }
-            } else {
-                LENS_CUDA(cudaMemsetAsync(polyA, 0, st.n_nodes * sizeof(dbl4), s));
-                LENS_CUDA(cudaMemsetAsync(polyC, 0, st.n_nodes * sizeof(double2), s));
-            }
-            { k_leafgrad<T><<<grid_for(st.n_nodes, TB), TB, 0, s>>>((uint32_t)st.n_nodes, st.link, (const T4*)st.nodeA,
-                                                                    (const T4*)st.exact0, (const T4*)st.exact1, st.kind,
-                                                                    polyA, polyC, gpart, st.perm,
-                                                                    (T*)g_species[si]); note_launch(); }
+            { k_leafgrad<T><<<grid_for(st.n_nodes, TB), TB, 0, s>>>(
+                (uint32_t)st.n_nodes, st.link, st.parent, (const T4*)st.nodeA, (const T4*)st.exact0, (const T4*)st.exact1,
+                st.kind, direct ? nullptr : adj, gpart, st.perm, (T*)g_species[si]); note_launch(); }
         }
         first = false;
         ++launches;
