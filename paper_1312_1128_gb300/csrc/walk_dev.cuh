@@ -78,7 +78,9 @@ template <int R, typename T> constexpr size_t cut_local_bytes() { return kCutSlo
 // it (a component that happens to be 1e-3 of the sum of |terms| otherwise
 // moves by 2e-5).
 struct SuperRec {
-    int ok;        // 1: use it; 0: each group starts at the root; 2: and takes no expansions of its own
+    // 1: use it; 0: each group starts at the root; 2: and takes no expansions
+    // of its own; 3 (of all records): as 2, in the plain kernel
+    int ok;
     int n;         // boxes left
     float hx, hy, cx, cy, id, pad;
     float h[kLocH];
@@ -1267,7 +1269,9 @@ template <typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int* stack
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const CutPool<T>& in = P.cut.in;
-    const int64_t n = in.cnt ? (int64_t)min(in.cnt[1], in.cap) : P.sub ? (int64_t)*P.sub_n : P.n_groups;
+    const int64_t n = in.cnt ? (int64_t)min(in.cnt[1], in.cap)
+                      : P.sub ? (int64_t)*P.sub_n
+                      : P.super && P.super[0].ok == 3 ? 0 : P.n_groups;
     for (;;) {
         uint32_t item = 0;
         if (lane == 0) item = atomicAdd(P.counter, 1u);
