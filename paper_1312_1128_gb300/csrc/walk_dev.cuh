@@ -744,10 +744,14 @@ template <int KIND, typename T, int R, bool AO, int TILE, bool LOC> struct WalkF
             local_finish(S.loc.sum, F);
             Eval E = eval(S);
             const float id = 1.0f / box_radius(E.box.z, E.box.w);
+            // (id = 0: a ray at infinity makes the box infinite.  Nothing is
+            // expanded then, and 0 * (x - inf) would be NaN for every ray)
+            if (id > 0.0f) {
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-                local_eval<AO>(F, (E.lx[r] - E.box.x) * id, (E.ly[r] - E.box.y) * id, id, E.part[r]);
-            E.fold();
+                for (int r = 0; r < R; ++r)
+                    local_eval<AO>(F, (E.lx[r] - E.box.x) * id, (E.ly[r] - E.box.y) * id, id, E.part[r]);
+                E.fold();
+            }
             __syncwarp();
         }
         if (n_halos > 0) eval(S).halos(halos, n_halos);

@@ -1,0 +1,55 @@
+"""Edge cases of the walk's forms: rays at infinity, faint lenses."""
+import numpy as np
+import pytest
+
+import lensgen
+import oracle
+from lens_testutil import comps_nfw, comps_points
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1312_1128_gb300 as L  # noqa: E402
+
+
+def cu(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def shoot(species, dx, dy, walk="warp", theta=0.3):
+    lens = L.Lens(species, theta=theta, group_rays=32, walk=walk)
+    o = lens.shoot(cu(dx), cu(dy))
+    lens.sync()
+    got = np.stack([x.double().cpu().numpy() for x in o], axis=1)
+    lens.close()
+    return got
+
+
+@pytest.mark.parametrize("kind", ["nfw", "points"])
+def test_infinite_ray(kind):
+    """A ray at infinity leaves the other rays of its group as they are: the
+    form without expansions as the reference, 1e-6 of the sum of |terms| (the
+    same terms in another order)."""
+    g = lensgen.rng(7)
+    if kind == "nfw":
+        p, n = lensgen.nfw_test_halos(3000, 22, 0.3), 1000
+        species, comps = [L.Species.nfw(cu(p), 3.0)], comps_nfw(p, 3.0)
+    else:
+        p, n = lensgen.point_disk(20000, 33), 16384 * 32 + 5  # (from 16,384 groups on: supergroups)
+        species, comps = [L.Species.points(cu(p))], comps_points(p)
+    dx, dy = (g.uniform(-0.9, 0.9, n).astype(np.float32) for _ in range(2))
+    dx[[3, n // 2]], dy[n - 1] = (np.inf, -np.inf), np.inf
+    got, ref = shoot(species, dx, dy), shoot(species, dx, dy, walk="pairs")
+    fin = np.isfinite(dx) & np.isfinite(dy)
+    assert np.isfinite(ref[fin]).all()
+    assert np.isfinite(got[fin]).all()
+    # (the rays that share a group with one at infinity are not known from
+    # outside: all of a small call, a sample of a large one)
+    idx = np.flatnonzero(fin)
+    if n > 2000:
+        idx = idx[lensgen.rng(3).integers(0, idx.size, 400)]
+    _, absum = oracle.direct_sum(comps, dx[idx].astype(np.float64), dy[idx].astype(np.float64), with_absum=True)
+    assert (np.abs(got[idx] - ref[idx]) / (absum + 1e-300)).max() <= 1e-6
