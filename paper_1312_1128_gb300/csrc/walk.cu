@@ -628,7 +628,7 @@ k_super(const __grid_constant__ WalkParams<float> P, const float* rcm, const uns
         }
         const float cx = 0.5f * (x0 + x1), cy = 0.5f * (y0 + y1);
         const float hx = fmaxf(x1 - cx, cx - x0) * 1.00001f, hy = fmaxf(y1 - cy, cy - y0) * 1.00001f;
-        const float d = box_radius(hx, hy), far2 = d * d * (1.0f / kLocRho2);
+        const float d = local_scale(hx, hy, P.nodeA[0].w), far2 = d * d * (1.0f / kLocRho2);
         if (lane == 0) stack[0] = 0;
         local_zero(S.loc.sum);
         __syncwarp();

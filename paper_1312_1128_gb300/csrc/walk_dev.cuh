@@ -234,6 +234,7 @@ template <typename T, int NR = 2> struct WalkTot {
 struct WalkLocal {
     LocalSum sum;
     float rho2;                // sources with (d/|w0|)^2 up to this are expanded
+    float d;                   // the expansion's scale (local_scale)
     uint8_t idx[2 * kBigCap];  // (buffers hold at most 256 entries)
 };
 struct NoLocal {};
@@ -644,7 +645,7 @@ template <int KIND, typename T, int R, bool AO, int TILE, bool LOC> struct WalkF
         if constexpr (LOC) {
             const int lane = threadIdx.x & 31;
             const float4 box = S.ray.box;
-            const float d = box_radius(box.z, box.w);
+            const float d = S.loc.d;
             LocalH H;
             H.zero();
             int nd = 0;
@@ -677,7 +678,7 @@ template <int KIND, typename T, int R, bool AO, int TILE, bool LOC> struct WalkF
         if constexpr (LOC) {
             const int lane = threadIdx.x & 31;
             const float4 box = S.ray.box;
-            const float d = box_radius(box.z, box.w);
+            const float d = S.loc.d;
             LocalH H;
             H.zero();
             int nd = 0;
@@ -743,7 +744,7 @@ template <int KIND, typename T, int R, bool AO, int TILE, bool LOC> struct WalkF
             LocalFields& F = *reinterpret_cast<LocalFields*>(S.buf.n0);  // (flushed: free)
             local_finish(S.loc.sum, F);
             Eval E = eval(S);
-            const float id = 1.0f / box_radius(E.box.z, E.box.w);
+            const float id = 1.0f / S.loc.d;
             // (id = 0: a ray at infinity makes the box infinite.  Nothing is
             // expanded then, and 0 * (x - inf) would be NaN for every ray)
             if (id > 0.0f) {
@@ -823,7 +824,10 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0, bool LOC = false> 
             for (int q = 0; q < (AO ? 2 : 5); ++q) S.tot.tot_s[q][r][lane] = S.tot.tot_c[q][r][lane] = T(0);
         if constexpr (LOC) {
             local_zero(S.loc.sum);
-            if (lane == 0) S.loc.rho2 = P.super && P.super[Cut->g / kSuperGroups].ok == 2 ? -1.0f : kLocRho2;
+            if (lane == 0) {
+                S.loc.rho2 = P.super && P.super[Cut->g / kSuperGroups].ok == 2 ? -1.0f : kLocRho2;
+                S.loc.d = local_scale(box.z, box.w, P.nodeA[0].w);
+            }
         }
         __syncwarp();
     }

@@ -53,3 +53,22 @@ def test_infinite_ray(kind):
         idx = idx[lensgen.rng(3).integers(0, idx.size, 400)]
     _, absum = oracle.direct_sum(comps, dx[idx].astype(np.float64), dy[idx].astype(np.float64), with_absum=True)
     assert (np.abs(got[idx] - ref[idx]) / (absum + 1e-300)).max() <= 1e-6
+
+
+@pytest.mark.parametrize("power", [-20, -40, -60])
+@pytest.mark.parametrize("n", [1, 2, 33])
+def test_unit_of_mass(power, n):
+    """The fields scale with the unit of mass, also for a group of one ray (a
+    call of one ray, the 33rd of a call, coincident rays): FP32 rounding does
+    not depend on a power of two, so the bar is a few roundings of each field
+    (1e-6 of the largest of its kind)."""
+    p = lensgen.nfw_test_halos(300, 22, 0.3)
+    q = p.copy()
+    q[:, 2] *= 2.0 ** power
+    if n == 2:
+        dx, dy = np.full(2, 0.37, np.float32), np.full(2, -0.11, np.float32)
+    else:
+        dx, dy = (lensgen.rng(5).uniform(-2.0, 2.0, n).astype(np.float32) for _ in range(2))
+    ref, got = shoot([L.Species.nfw(cu(p), 3.0)], dx, dy), shoot([L.Species.nfw(cu(q), 3.0)], dx, dy) * 2.0 ** -power
+    scale = np.abs(ref).max(axis=1, keepdims=True)
+    assert (np.abs(got - ref) / scale).max() <= 1e-6
