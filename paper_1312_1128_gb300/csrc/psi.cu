@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
             g = __shfl_sync(full, g, 0);
             if ((int64_t)g >= P.n_groups) break;
         } else {
-            if (!next_item(P, stack, S.cut)) break;
+            if (!next_item<R>(P, stack, S.cut)) break;
             g = S.cut.g;
         }
         const bool head = DIRECT || S.cut.item == kNoItem;  // the group's first (or only) item
@@ -406,11 +406,14 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
                 C.flush_near();
                 C.flush_big();
                 if (P.n_halos > 0 && head && S.cut.seg == 0) C.halos();
+                // (a part's cut counts from its own start)
+                count_item(C, g, P.grange[g].y, head && S.cut.seg == 0);
+                C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
             } while (S.cut.local && local_next_part<R, 3>(P.cut, S.cut, stack, [&](int r, int q) {
                          return C.tot_s[r][q] + C.tot_c[r][q]; }));
         }
         __syncwarp();
-        count_item(C, g, rg.y, head);
+        if constexpr (DIRECT) count_item(C, g, rg.y, head);
         T* tot = DIRECT ? nullptr : item_totals<R>(P.cut, S.cut);
 #pragma unroll
         for (int r = 0; r < R; ++r) {

@@ -390,7 +390,7 @@ walk_kernel(const __grid_constant__ WalkParams<T> P)
             slice = item % (uint32_t)NS;
             g = item / (uint32_t)NS;
         } else {
-            if (!next_item(P, stack, S.cut)) break;
+            if (!next_item<R>(P, stack, S.cut)) break;
             g = S.cut.g;
         }
         // the group's first (or only) item
@@ -436,12 +436,15 @@ walk_kernel(const __grid_constant__ WalkParams<T> P)
                     }
                 }
                 Ctx::Flush::finish(P.halos, first ? P.n_halos : 0, sr, delta);
+                // (a part's cut counts from its own start)
+                count_item(C, g, P.grange[g].y, first);
+                C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
             } while (S.cut.local && local_next_part<R, AO ? 2 : 5>(P.cut, S.cut, stack,
                                                                    [&](int r, int q) { return C.total(r, q); }));
         }
         __syncwarp();
         const uint2 rg = P.grange[g];
-        count_item(C, g, rg.y, head);
+        if constexpr (DIRECT) count_item(C, g, rg.y, head);
 
         T* tot = DIRECT ? nullptr : item_totals<R>(P.cut, S.cut);
 #pragma unroll

@@ -19,10 +19,14 @@ namespace lens {
 // groups leaves most of the chip idle (295 groups of a 97^2-ray map: 2.9 ms
 // for 295 warps of 3,648), and a group over a density cusp runs alone at the
 // end of a launch of many (walk_rounds says when groups are cut).  Every item
-// writes its rays' totals to a slot; k_cut_sum adds the slots of a group in
-// order.  Where a cut finds its pool full, the warp itself walks the parts one
-// after another and adds their totals in the same order: the bits do not
-// depend on which warp ran what.
+// writes its rays' totals to a place of its own; k_cut_sum adds those of a
+// group in order.
+//
+// The bits do not depend on which warp ran what.  Where a cut finds its pool
+// full, the warp itself walks the parts one after another, cuts them again
+// where a part of the pool would be, and adds all totals in the same order.
+// The number of parts is fixed then; only where the pool has room for every
+// group does it follow from how many are cut.
 constexpr int kCutNodes = 384;   // boxes handed over per cut
 constexpr int kCutRanges = 96;   // deferred big lists per cut
 constexpr int kLongList = 8;     // chunks of a big list that is deferred wherever a group may be cut
@@ -30,26 +34,28 @@ constexpr uint32_t kNoItem = 0xffffffffu, kNoCut = 0xffffffffu;
 
 struct alignas(16) CutSlot {
     uint32_t g;        // group
-    uint32_t base;     // its totals: slot base (before the cut), base + 1 + j (part j)
-    uint32_t parts;    // 0: not cut after all
     uint32_t n_nodes, n_ranges;
-    int32_t parent;    // the totals go to this slot of the pool before, or -1: the outputs
-    uint32_t pad[2];
+    int32_t parent;    // the totals go to this part of the pool before, or -1: the outputs
     int2 ranges[kCutRanges];  // big lists {first entry, entries}
     int nodes[kCutNodes];
 };
 
 static_assert(sizeof(CutSlot) == kCutSlotBytes, "scratch layout");
 
-// The cuts of one launch: cnt[0] counts cuts, cnt[1] item slots.  Every slot
-// below min(cnt[1], cap) is written by the cut that took it: item[base] =
-// kNoItem, item[base + 1 + j] = cut << 7 | j.
+// The cuts of one launch.
 template <typename T> struct CutPool {
-    uint32_t* cnt = nullptr;
+    uint32_t* cnt = nullptr;  // cuts made (above max_cuts: by their own warp)
     CutSlot* slots = nullptr;
-    uint32_t max_cuts = 0, cap = 0;
-    uint32_t* item = nullptr;
-    T* part = nullptr;      // cap x 5 x 32R totals
+    uint32_t max_cuts = 0;
+    uint32_t parts = 0;     // parts per cut
+    uint32_t items = 0;     // if not 0: fewer parts, so that there are at most these in all
+    T* head = nullptr;      // max_cuts x 5 x 32R totals: of the walk up to the cut
+    T* part = nullptr;      // of part j of cut i: (i x parts + j) x 5 x 32R
+    LENS_DEV uint32_t cuts() const { return min(*cnt, max_cuts); }
+    LENS_DEV uint32_t parts_of(uint32_t n_cuts) const
+    {
+        return items == 0 || n_cuts == 0 ? parts : max(1u, min(parts, items / n_cuts));
+    }
 };
 
 template <typename T> struct CutParams {
@@ -57,10 +63,14 @@ template <typename T> struct CutParams {
     CutPool<T> out;         // where this launch's cuts go (null: no cuts)
     uint32_t limit = 0;     // evaluated entries before a group is cut
     uint32_t limit_stretched = 0;  // the same for a stretched group (0: as the others)
-    uint32_t parts = 0;
+    uint32_t few_parts = 0;    // parts of cuts into fewer than this are cut again at 4 x limit
     int min_nodes = 0;      // boxes on the stack to be worth a cut
     int defer = 0;          // every big list met before the cut goes to the parts
     unsigned char* local = nullptr;  // per warp: deferred lists, and a cut's slot and sums if its pool is full
+    size_t local_bytes = 0;          // of one warp: cut_local_bytes, twice where its parts may be cut too
+    // the cuts of parts that the warp walks itself (as in the next launch)
+    uint32_t again_limit = kNoCut, again_parts = 0;
+    int again_min_nodes = 0;
 };
 
 template <int R, typename T> constexpr size_t cut_local_bytes() { return kCutSlotBytes + 2 * 5 * 32 * R * sizeof(T); }
@@ -198,7 +208,7 @@ template <int KIND, typename T, int TILE = 0> struct WalkBuf {
 struct WalkCut {
     // the item
     uint32_t g;          // group
-    uint32_t item;       // the part's slot of the in pool (kNoItem: a whole group)
+    uint32_t item;       // the part's place in the in pool (kNoItem: a whole group)
     int sp;              // boxes on the stack
     const CutSlot* cs;   // the cut it is a part of, or null
     int j, parts;        // part j of parts
@@ -211,8 +221,10 @@ struct WalkCut {
     uint32_t chunks;     // their chunks
     int fired;           // was cut
     int local;           // the parts are walked here (the pool was full)
-    uint32_t base;       // the cut's first item slot
+    uint32_t cut;        // its place in the out pool
     int seg;             // local: the part being walked
+    int sub, seg2;       // that part was cut too: its subpart being walked
+    CutSlot* own;        // the warp's place for what is cut or put aside now
 };
 
 // The list ranges of one traversal step (one per lane) and the Neumaier-
@@ -1056,36 +1068,26 @@ LENS_DEV void append_big(Ctx& C, int cnt, int z, int w, int c0 = 0, int cstep = 
 
 
 // The warp's own cut slot (the lists deferred so far, and the boxes of a cut
-// whose pool is full) and the sums beside it.
-template <int R, typename T> LENS_DEV unsigned char* cut_own(const CutParams<T>& cp)
+// whose pool is full) and the sums beside it; level 1: of a part's cut.
+template <int R, typename T> LENS_DEV unsigned char* cut_own(const CutParams<T>& cp, int level = 0)
 {
     const int64_t w = (int64_t)blockIdx.x * kWalkWarps + (threadIdx.x >> 5);
-    return cp.local + w * (int64_t)cut_local_bytes<R, T>();
+    return cp.local + w * (int64_t)cp.local_bytes + level * (int64_t)cut_local_bytes<R, T>();
 }
 
 // Cut the walk: the boxes at the bottom of the stack (the shallowest) and the
 // deferred lists go to a slot of the pool, or stay in the warp's own if the
-// pool is full (1 + parts item slots are taken; those below the pool's end
-// are written whatever comes of it).  Returns how many boxes stay (at the
-// bottom of the stack).
+// pool is full.  Returns how many boxes stay (at the bottom of the stack).
 template <int R, typename T> LENS_DEV int cut_now(const CutParams<T>& cp, WalkCut& K, int* stack, int sp)
 {
-    const unsigned full = 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31;
     const CutPool<T>& pool = cp.out;
-    uint32_t ci = 0, base = 0;
-    if (lane == 0) ci = atomicAdd(pool.cnt, 1u);
-    ci = __shfl_sync(full, ci, 0);
-    bool pooled = ci < pool.max_cuts;
-    if (pooled) {
-        if (lane == 0) base = atomicAdd(pool.cnt + 1, cp.parts + 1);
-        base = __shfl_sync(full, base, 0);
-        pooled = base + cp.parts + 1 <= pool.cap;
-        for (uint32_t j = lane; j < cp.parts + 1; j += 32)
-            if (base + j < pool.cap) pool.item[base + j] = pooled && j > 0 ? (ci << 7 | (j - 1)) : kNoItem;
-        if (!pooled && lane == 0) pool.slots[ci].parts = 0;
-    }
-    CutSlot* own = (CutSlot*)cut_own<R>(cp);
+    const bool part = K.local;  // a part that the warp walks itself
+    uint32_t ci = 0;
+    if (lane == 0 && !part) ci = atomicAdd(pool.cnt, 1u);
+    ci = __shfl_sync(0xffffffffu, ci, 0);
+    const bool pooled = !part && ci < pool.max_cuts;
+    CutSlot* own = K.own;
     CutSlot* s = pooled ? pool.slots + ci : own;
     const int nd = sp < kCutNodes ? sp : kCutNodes;
     if (pooled)
@@ -1093,14 +1095,17 @@ template <int R, typename T> LENS_DEV int cut_now(const CutParams<T>& cp, WalkCu
     for (int i = (int)lane; i < nd; i += 32) s->nodes[i] = stack[i];
     if (lane == 0) {
         s->g = K.g;
-        s->base = base;
-        s->parts = cp.parts;
         s->n_nodes = (uint32_t)nd;
         s->n_ranges = (uint32_t)K.n_ranges;
         s->parent = K.item == kNoItem ? -1 : (int32_t)K.item;
-        K.fired = 1;
-        K.local = !pooled;
-        K.base = base;
+        if (part) {
+            K.sub = 1;
+            K.seg2 = 0;
+        } else {
+            K.fired = 1;
+            K.local = !pooled;
+            K.cut = ci;
+        }
     }
     __syncwarp();
     for (int i = nd; i < sp; i += 32) {
@@ -1146,7 +1151,7 @@ LENS_DEV bool traverse(Ctx& C, int* stack, int sp)
                 } else {
                     rn = C.Cut->n_ranges;
                     if (lane == 0) {
-                        C.Cut->rs = ((CutSlot*)cut_own<Ctx::kR>(P.cut))->ranges;
+                        C.Cut->rs = C.Cut->own->ranges;
                         C.Cut->j = 0;
                         C.Cut->parts = 1;
                     }
@@ -1224,7 +1229,7 @@ LENS_DEV bool traverse(Ctx& C, int* stack, int sp)
                         const int n0 = C.Cut->n_ranges, pos = n0 + __popc(bm & ((1u << lane) - 1u));
                         uint32_t ch = 0;
                         if (put && pos < kCutRanges) {
-                            ((CutSlot*)cut_own<Ctx::kR>(P.cut))->ranges[pos] = make_int2(Lk.z, Lk.w);
+                            C.Cut->own->ranges[pos] = make_int2(Lk.z, Lk.w);
                             ch = (uint32_t)cnt;
                             cnt = 0;
                         }
@@ -1272,12 +1277,13 @@ LENS_DEV void load_part(WalkCut& K, int* stack)
 }
 
 // Take the next item (false: none left); its boxes go on the stack.
-template <typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int* stack, WalkCut& K)
+template <int R, typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int* stack, WalkCut& K)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const CutPool<T>& in = P.cut.in;
-    const int64_t n = in.cnt ? (int64_t)min(in.cnt[1], in.cap)
+    const uint32_t cuts = in.cnt ? in.cuts() : 0u, parts = in.parts_of(cuts);
+    const int64_t n = in.cnt ? (int64_t)cuts * parts
                       : P.sub ? (int64_t)*P.sub_n
                       : P.super && P.super[0].ok == 3 ? 0 : P.n_groups;
     for (;;) {
@@ -1285,26 +1291,21 @@ template <typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int* stack
         if (lane == 0) item = atomicAdd(P.counter, 1u);
         item = __shfl_sync(full, item, 0);
         if ((int64_t)item >= n) return false;
-        uint32_t e = 0;
-        if (in.cnt) {
-            e = in.item[item];
-            if (e == kNoItem) continue;
-        } else if (P.skip && P.gflag[P.order ? P.order[item] : item]) {
-            continue;
-        }
+        if (!in.cnt && P.skip && P.gflag[P.order ? P.order[item] : item]) continue;
         if (lane == 0) {
-            K.limit = P.cut.out.cnt ? P.cut.limit : kNoCut;
+            K.limit = !P.cut.out.cnt ? kNoCut : P.cut.limit << (parts < P.cut.few_parts ? 2 : 0);
             K.min_nodes = P.cut.min_nodes;
             K.n_ranges = 0;
             K.chunks = 0;
             K.fired = K.local = 0;
-            K.seg = 0;
+            K.seg = K.sub = 0;
+            K.own = (CutSlot*)cut_own<R>(P.cut);
             K.rn = 0;
             if (in.cnt) {
-                const CutSlot* cs = in.slots + (e >> 7);
+                const CutSlot* cs = in.slots + item / parts;
                 K.cs = cs;
-                K.j = (int)(e & 127u);
-                K.parts = (int)cs->parts;
+                K.j = (int)(item % parts);
+                K.parts = (int)parts;
                 K.g = cs->g;
                 K.item = item;
             } else {
@@ -1334,37 +1335,64 @@ template <typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int* stack
     }
 }
 
-// A cut whose pool was full: after each segment (the group's own, then each
-// part) its totals are added to the sums beside the warp's slot, as k_cut_sum
-// adds them; then the next part's boxes go on the stack.  False: no part left.
+// A cut whose pool was full: after each segment (the item's own, then each
+// part; after a part that was cut too, each of its subparts) its totals are
+// added to the sums beside the warp's slot, as k_cut_sum adds them; then the
+// next part's boxes go on the stack.  False: no part left.
 template <int R, int NQ, typename T, class Tot>
 LENS_DEV bool local_next_part(const CutParams<T>& cp, WalkCut& K, int* stack, Tot&& tot)
 {
-    const int lane = threadIdx.x & 31, seg = K.seg;
-    unsigned char* own = cut_own<R>(cp);
-    T* sums = (T*)(own + kCutSlotBytes);
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            T* a = sums + ((q * R + r) * 2) * 32 + lane;
-            T s = seg ? a[0] : tot(r, q), c = seg ? a[32] : T(0);
-            if (seg) Comp5<T>::add1(s, c, tot(r, q));
-            a[0] = s;
-            a[32] = c;
+    const int lane = threadIdx.x & 31;
+    auto at = [&](int level, int r, int q) {
+        return (T*)(cut_own<R>(cp, level) + kCutSlotBytes) + ((q * R + r) * 2) * 32 + lane;
+    };
+    auto next = [&](int level, int j, uint32_t parts) {
+        if (lane == 0) {
+            K.cs = (CutSlot*)cut_own<R>(cp, level);
+            K.j = j;
+            K.parts = (int)parts;
+            K.own = (CutSlot*)cut_own<R>(cp, 1);
+            K.n_ranges = 0;
+            K.chunks = 0;
+            K.limit = level ? kNoCut : cp.again_limit;
+            K.min_nodes = cp.again_min_nodes;
+            if (level) {
+                K.seg2 = j + 1;
+            } else {
+                K.seg = j + 1;
+                K.sub = 0;
+            }
         }
-    __syncwarp();
-    if (seg == (int)cp.parts) return false;
-    if (lane == 0) {
-        K.cs = (CutSlot*)own;
-        K.j = seg;
-        K.parts = (int)cp.parts;
-        K.seg = seg + 1;
-        K.limit = kNoCut;
+        __syncwarp();
+        load_part(K, stack);
+    };
+    const int seg = K.seg, sub = K.sub, seg2 = K.seg2;
+    for (int level = sub; level >= 0; --level) {
+        const bool first = (level ? seg2 : seg) == 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                T* a = at(level, r, q);
+                T v = tot(r, q);
+                if (sub && level == 0) {
+                    const T* b = at(1, r, q);
+                    v = b[0] + b[32];
+                }
+                T x = first ? v : a[0], c = first ? T(0) : a[32];
+                if (!first) Comp5<T>::add1(x, c, v);
+                a[0] = x;
+                a[32] = c;
+            }
+        __syncwarp();
+        const int j = level ? seg2 : seg;
+        const uint32_t parts = level ? cp.again_parts : cp.out.parts;
+        if (j < (int)parts) {
+            next(level, j, parts);
+            return true;
+        }
     }
-    __syncwarp();
-    load_part(K, stack);
-    return true;
+    return false;
 }
 template <int R, typename T> LENS_DEV T local_total(const CutParams<T>& cp, int r, int q)
 {
@@ -1372,11 +1400,11 @@ template <int R, typename T> LENS_DEV T local_total(const CutParams<T>& cp, int 
     return a[0] + a[32];
 }
 
-// Where an item's totals go: the outputs (null), its own slot, or, when it was
-// cut, the cut's first slot.
+// Where an item's totals go: the outputs (null), its own place in its pool,
+// or, when it was cut, the cut's.
 template <int R, typename T> LENS_DEV T* item_totals(const CutParams<T>& cp, const WalkCut& K)
 {
-    if (K.fired && !K.local) return cp.out.part + (int64_t)K.base * (5 * 32 * R);
+    if (K.fired && !K.local) return cp.out.head + (int64_t)K.cut * (5 * 32 * R);
     if (K.item != kNoItem) return cp.in.part + (int64_t)K.item * (5 * 32 * R);
     return nullptr;
 }
@@ -1400,26 +1428,28 @@ template <class Ctx> LENS_DEV void count_item(const Ctx& C, uint32_t g, uint32_t
 }
 
 // The totals of every cut group of `pool`, its parts added in order with
-// Neumaier compensation, into the outputs, or into the slot of the part that
+// Neumaier compensation, into the outputs, or into the place of the part that
 // was cut again (`to`).  One warp per (cut, component).
 template <typename T, int R>
 __global__ void k_cut_sum(CutPool<T> pool, CutPool<T> to, WalkParams<T> P, int nq)
 {
     const int lane = threadIdx.x & 31;
-    const uint32_t nc = min(pool.cnt[0], pool.max_cuts) * (uint32_t)nq;
+    const uint32_t cuts = pool.cuts(), nc = cuts * (uint32_t)nq;
+    const int parts = (int)pool.parts_of(cuts);
     const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
     constexpr int64_t stride = 5 * 32 * R;
     for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nc; w += nw) {
-        const CutSlot& cs = pool.slots[w / (uint32_t)nq];
-        const int q = (int)(w % (uint32_t)nq), parts = (int)cs.parts;
-        if (parts == 0) continue;
+        const uint32_t ci = w / (uint32_t)nq;
+        const CutSlot& cs = pool.slots[ci];
+        const int q = (int)(w % (uint32_t)nq);
         const uint2 rg = P.grange[cs.g];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const T* p = pool.part + (int64_t)cs.base * stride + (q * R + r) * 32 + lane;
-            T s = p[0], c = T(0);
+            const int64_t at = (q * R + r) * 32 + lane;
+            const T* p = pool.part + (int64_t)ci * parts * stride + at;
+            T s = pool.head[(int64_t)ci * stride + at], c = T(0);
 #pragma unroll 8
-            for (int j = 1; j <= parts; ++j) Comp5<T>::add1(s, c, p[j * stride]);
+            for (int j = 0; j < parts; ++j) Comp5<T>::add1(s, c, p[j * stride]);
             T val = s + c;
             if (cs.parent >= 0) {
                 to.part[(int64_t)cs.parent * stride + (q * R + r) * 32 + lane] = val;
@@ -1443,64 +1473,81 @@ __global__ void k_cut_sum(CutPool<T> pool, CutPool<T> to, WalkParams<T> P, int n
 //     launch's warps.
 //   above: only a group far heavier than the others (16,384 entries and more;
 //     an average one evaluates 5,000 to 7,000), or a stretched one (which may
-//     hold most of the tree) beyond 8,192.
+//     hold most of the tree) beyond 8,192; the fewer they are, the more parts.
+//     Where the groups are more than the pool has room for, 8 parts each.
 //   keep_order (FP32 point masses): none but the heavy ones.  Over a patch much
 //     smaller than the distances all rays share the rounding of one sum of
 //     thousands of terms, which shows in a component that happens to be small
 //     (1e-3 of the sum of |terms|): such groups keep their order of summation.
-// Which groups are cut depends on their own walk alone.
 template <typename T, int R, typename Walk>
 void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& L, uint32_t* counter, Walk&& walk,
                  cudaStream_t s, bool keep_order = false)
 {
     // counter: 8 words, zeroed by the caller: work counters, then each pool's
     CutPool<T> pool[2];
-    char *slot = base + L.cut_slot, *item = base + L.cut_item, *part = base + L.cut_part;
-    for (int k = 0; k < 2; ++k) {
-        pool[k].cnt = counter + 4 + 2 * k;
-        pool[k].slots = (CutSlot*)slot;
-        pool[k].max_cuts = kCutMax[k];
-        pool[k].item = (uint32_t*)item;
-        pool[k].part = (T*)part;
-        const size_t fit = kCutItems[k] * kCutPartBytes / (5 * 32 * R * sizeof(T));
-        pool[k].cap = (uint32_t)(fit < kCutItems[k] ? fit : kCutItems[k]);
-        slot += kCutMax[k] * kCutSlotBytes;
-        item += kCutItems[k] * sizeof(uint32_t);
-        part += kCutItems[k] * kCutPartBytes;
+    constexpr size_t total = 5 * 32 * R * sizeof(T);
+    char* at = base + L.cut;
+    auto take = [&](size_t bytes) {
+        char* p = at;
+        at += (bytes + 255) & ~(size_t)255;
+        return p;
+    };
+    const size_t local_bytes = cut_local_bytes<R, T>() * 2;
+    unsigned char* local = (unsigned char*)take(L.cut_warps * local_bytes);
+    // the second pool: parts that are cut again
+    pool[1].parts = ng <= 4096 && !keep_order ? 16 : 32;
+    pool[1].max_cuts = (uint32_t)(kCutAgainBytes / (pool[1].parts * total));
+    pool[1].slots = (CutSlot*)take(pool[1].max_cuts * sizeof(CutSlot));
+    pool[1].head = (T*)take(pool[1].max_cuts * total);
+    pool[1].part = (T*)take(pool[1].max_cuts * pool[1].parts * total);
+    // the first has the rest: every group that may be cut has a place
+    const size_t room = L.cut_bytes - (size_t)(at - (base + L.cut)) - 4 * 256;
+    const bool few = ng <= 4096 && !keep_order;
+    bool all = true;
+    if (few) {
+        const size_t fit = (room - (size_t)ng * (sizeof(CutSlot) + total)) / total;
+        pool[0].max_cuts = (uint32_t)ng;
+        pool[0].parts = ng <= 512 ? 64 : 16;
+        pool[0].items = (uint32_t)std::min<size_t>(ng <= 512 ? 8192 : 28672, fit);
+    } else {
+        // a place for every group, or 8 parts each for as many as fit
+        all = (size_t)ng * (sizeof(CutSlot) + 2 * total) <= room;
+        pool[0].max_cuts = (uint32_t)(all ? (size_t)ng : room / (sizeof(CutSlot) + 9 * total));
+        pool[0].parts = all ? 32 : 8;
+        pool[0].items = all ? (uint32_t)std::min<size_t>(28672, (room - pool[0].max_cuts * (sizeof(CutSlot) + total)) / total) : 0;
     }
+    pool[0].slots = (CutSlot*)take(pool[0].max_cuts * sizeof(CutSlot));
+    pool[0].head = (T*)take(pool[0].max_cuts * total);
+    pool[0].part = (T*)take((all ? (size_t)std::max(pool[0].max_cuts, pool[0].items) : (size_t)pool[0].max_cuts * 8) * total);
+    for (int k = 0; k < 2; ++k) pool[k].cnt = counter + 4 + k;
     constexpr int rounds = 3;
     CutParams<T> c[rounds];
     P.gflag = (const uint8_t*)(base + L.gflag);
-    if (ng <= 512 && !keep_order) {
-        const int64_t want = 8192 / (ng > 0 ? ng : 1);
-        c[0].parts = (uint32_t)(want < 16 ? 16 : want > 64 ? 64 : want);
+    if (few && ng <= 512) {
         c[0].limit = 0;
         c[0].min_nodes = 64;
         c[0].defer = 1;
-        c[1].parts = 16;
         c[1].limit = 512;
         c[1].min_nodes = 16;
-    } else if (ng <= 4096 && !keep_order) {
-        // (every group may be cut without filling the pool: a part walked by
-        // the group's own warp is not cut again, one of the pool may be)
-        const uint32_t fit = pool[0].cap / (uint32_t)ng - 1;
-        c[0].parts = fit < 16 ? fit : 16;
+    } else if (few) {
         c[0].limit = (uint32_t)(ng / 4 + 256);
         c[0].min_nodes = 32;
-        c[1].parts = 16;
         c[1].limit = c[0].limit;
         c[1].min_nodes = 16;
     } else {
-        c[0].parts = 8;
         c[0].limit = (uint32_t)(ng <= 10922 || keep_order ? 16384 : 3 * (ng / 2));
         c[0].limit_stretched = 8192;
         c[0].min_nodes = 32;
-        c[1].parts = 32;
         c[1].limit = 8192;
+        c[1].few_parts = 4;  // (thousands of cuts fill the chip by themselves: only the heaviest again)
         c[1].min_nodes = 16;
     }
+    c[0].again_limit = c[1].limit << (pool[0].parts < c[1].few_parts ? 2 : 0);
+    c[0].again_parts = pool[1].parts;
+    c[0].again_min_nodes = c[1].min_nodes;
     for (int r = 0; r < rounds; ++r) {
-        c[r].local = (unsigned char*)(base + L.cut_local);
+        c[r].local = local;
+        c[r].local_bytes = local_bytes;
         P.counter = counter + r;
         if (r > 0) c[r].in = pool[r - 1];
         if (r + 1 < rounds) c[r].out = pool[r];
@@ -1508,7 +1555,7 @@ void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& 
         walk(P);
     }
     for (int r = rounds - 2; r >= 0; --r) {
-        const int64_t most = r > 0 || kCutMax[r] < ng ? kCutMax[r] : ng;
+        const int64_t most = std::min<int64_t>(pool[r].max_cuts, r > 0 ? 2048 : ng);
         k_cut_sum<T, R><<<(unsigned)((most * nq + 7) / 8), 256, 0, s>>>(pool[r], r > 0 ? pool[r - 1] : CutPool<T>{}, P, nq);
         note_launch();
     }

@@ -44,14 +44,16 @@ LENS_DEV bool box_reaches_group(const vec4_t<T>& b, const v2_t<T>& H, const vec4
 
 struct Layout {
     size_t boff, borig, gfirst, bbox, k0, k1, v0, v1, tmp, rl, ridx, gH, gbox, grange, counter,
-        stack, split, gcost, heavy, cut_slot, cut_item, cut_part, cut_local, super, sdelta, gflag, sub, total;
+        stack, split, gcost, heavy, cut, super, sdelta, gflag, sub, total;
+    size_t cut_bytes;   // of the region at cut
+    size_t cut_warps;   // warps of a tree walk that have a place of their own there
 };
 
-// Cut groups (walk_dev.cuh): two pools, for the cuts of a call's first launch
-// and of its second; slots of kCutSlotBytes, item slots, and totals of
-// 5 x 32 R values per item slot.
-constexpr uint32_t kCutMax[2] = {4096, 2048}, kCutItems[2] = {32768, 16384};
-constexpr size_t kCutSlotBytes = 2336;
+// Cut groups (walk_dev.cuh): one region for a call's cuts, split by the walk
+// (walk_rounds): a place for each of its warps, then two pools.
+constexpr size_t kCutBytes = (size_t)112 << 20;       // the whole region
+constexpr size_t kCutAgainBytes = (size_t)20 << 20;   // totals of the second pool's parts
+constexpr size_t kCutSlotBytes = 2320;
 // Stretched groups: Morton order jumps between quadrants, so unless the rays
 // fill power-of-two squares a few groups span half the map and open most of
 // the tree (one warp then walked on for 18 of 20 ms at 700^2 rays through 3e5
@@ -66,7 +68,6 @@ constexpr float kStretch = 16.0f;
 constexpr int kSuperGroups = 32;
 constexpr size_t kSuperBytes = 1664;
 constexpr int kCutBlocks = 8;  // resident blocks per SM of a tree walk (each warp has its own slot and sums)
-constexpr size_t kCutPartBytes = 5 * 64 * 4;  // per item slot (R = 2 in FP32); fewer item slots fit wider totals
 
 // Tags of a kept interaction-list entry (LENS_KEEP_LISTS): the box's index
 // in the low 29 bits; a box may be accepted (far cell) or an opened leaf, and
@@ -110,11 +111,9 @@ inline Layout make_layout(int64_t n, int64_t nb, int64_t slots)
     L.split = o; o += al(split_values(slots) * 5 * sizeof(double));
     L.gcost = o; o += al(ng * sizeof(uint32_t));
     L.heavy = o; o += al(64 + (size_t)kHeavyItems * sizeof(uint32_t));
-    L.cut_slot = o; o += al((kCutMax[0] + kCutMax[1]) * kCutSlotBytes);
-    L.cut_item = o; o += al((kCutItems[0] + kCutItems[1]) * sizeof(uint32_t));
-    L.cut_part = o; o += al((kCutItems[0] + kCutItems[1]) * kCutPartBytes);
-    // (slots = 16 blocks per SM x kWalkWarps; sums of 5 x 128 FP32 or 64 FP64 values and their corrections)
-    L.cut_local = o; o += al((size_t)slots / 16 * kCutBlocks * (kCutSlotBytes + 2 * 5 * 128 * sizeof(float)));
+    L.cut = o; o += al(kCutBytes);
+    L.cut_bytes = kCutBytes;
+    L.cut_warps = (size_t)slots / 16 * kCutBlocks;  // (slots: 16 blocks per SM)
     L.super = o; o += al((size_t)(ng / kSuperGroups + 1) * kSuperBytes);
     L.sdelta = o; o += al(ng * 4 * sizeof(float));
     L.gflag = o; o += al(ng);

@@ -72,3 +72,25 @@ def test_unit_of_mass(power, n):
     ref, got = shoot([L.Species.nfw(cu(p), 3.0)], dx, dy), shoot([L.Species.nfw(cu(q), 3.0)], dx, dy) * 2.0 ** -power
     scale = np.abs(ref).max(axis=1, keepdims=True)
     assert (np.abs(got - ref) / scale).max() <= 1e-6
+
+
+@pytest.mark.parametrize("call", ["shoot", "potential"])
+@pytest.mark.parametrize("kind,theta", [("points", 0.01), ("gauss", 0.01), ("nfw", 0.01)])
+def test_repeated_call_is_bitwise_equal_when_most_groups_are_cut(kind, theta, call):
+    """8,450 groups, most of them above the limit of a cut (16,384 entries):
+    more cuts than could all have several parts of their own."""
+    p = lensgen.nfw_particles(60_000, 9, nsph=32)
+    if kind == "nfw":
+        p[:, 3] = 0.01
+    species = L.Species.points(cu(p)) if kind == "points" else getattr(L.Species, kind)(cu(p), 3.0)
+    lens = L.Lens([species], theta=theta, group_rays=32)
+    rx, ry = lensgen.grid_rays(520, -1.0, 1.0, dtype=np.float32)
+    dx, dy = cu(rx), cu(ry)
+    run = lens.shoot if call == "shoot" else lens.potential
+    lens.shoot(dx, dy, flags=L.COUNT)
+    c = lens.counters()
+    assert c["cells"] // 2 + c["leaf_particles"] + c["big_kept"] > 16384 * c["groups"]
+    first = [o.clone() for o in run(dx, dy)]
+    for _ in range(5):
+        assert all(torch.equal(a, b) for a, b in zip(first, run(dx, dy)))
+    lens.close()
