@@ -93,14 +93,14 @@ LENS_DEV float box_radius(float hx, float hy)
 }
 
 // Scale d of a group's expansion: its half diagonal, but at least an FP32
-// rounding (2^-24) of the root's r_cut (rcut2: its square).  A group of one ray
+// rounding (2^-24) of the root's r_cm.  A group of one ray
 // has a half diagonal of 1e-30; the coefficient of zeta is then d m / w^2, below
 // the normal numbers for m / w^2 < 1e-8, and its quotient by d, gamma, is lost.
 // Sources nearer than d / 0.18 are evaluated ray by ray, so a larger d only
 // makes the expansion's remainder smaller.
-LENS_DEV float local_scale(float hx, float hy, float rcut2)
+LENS_DEV float local_scale(float hx, float hy, float root_rcm)
 {
-    return fmaxf(box_radius(hx, hy), 5.9604645e-8f * sqrtf(rcut2));
+    return fmaxf(box_radius(hx, hy), 5.9604645e-8f * root_rcm);
 }
 
 // A lane's share of h.

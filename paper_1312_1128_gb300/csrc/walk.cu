@@ -631,7 +631,7 @@ k_super(const __grid_constant__ WalkParams<float> P, const float* rcm, const uns
         }
         const float cx = 0.5f * (x0 + x1), cy = 0.5f * (y0 + y1);
         const float hx = fmaxf(x1 - cx, cx - x0) * 1.00001f, hy = fmaxf(y1 - cy, cy - y0) * 1.00001f;
-        const float d = local_scale(hx, hy, P.nodeA[0].w), far2 = d * d * (1.0f / kLocRho2);
+        const float d = local_scale(hx, hy, rcm[0]), far2 = d * d * (1.0f / kLocRho2);
         if (lane == 0) stack[0] = 0;
         local_zero(S.loc.sum);
         __syncwarp();
@@ -1265,6 +1265,7 @@ static lens_status enqueue_typed(lens_tree* t, const ShootPlan& plan, const void
         P.nodeA = (const T4*)st.nodeA;
         P.nodeB = (const T2*)st.nodeB;
         P.link = st.link;
+        P.node_rcm = st.node_rcm;
         P.leaf0 = (const T4*)((direct || st.kind == LENS_POINT) ? st.exact0 : st.leaf0);
         P.leaf1 = (const T4*)st.exact1;
         P.big0 = (const T4*)st.big0;

@@ -107,6 +107,7 @@ template <typename T> struct WalkParams : EvalConsts<T> {
     const vec4_t<T>* nodeA;
     const v2_t<T>* nodeB;
     const int4* link;
+    const float* node_rcm;
     const vec4_t<T>* leaf0;   // near records (listed particles marked)
     const vec4_t<T>* leaf1;   // NFW second record
     const vec4_t<T>* big0;       // {x, y, s^2, r0^2}
@@ -838,7 +839,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0, bool LOC = false> 
             local_zero(S.loc.sum);
             if (lane == 0) {
                 S.loc.rho2 = P.super && P.super[Cut->g / kSuperGroups].ok == 2 ? -1.0f : kLocRho2;
-                S.loc.d = local_scale(box.z, box.w, P.nodeA[0].w);
+                S.loc.d = local_scale(box.z, box.w, P.node_rcm[0]);
             }
         }
         __syncwarp();
