@@ -436,8 +436,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
     }
 }
 
-template <int KIND, typename T, int R, bool DIRECT>
-static void psi_launch_one(const WalkParams<T>& P, const PsiConsts<T>& K, int num_sms, cudaStream_t s)
+template <int KIND, typename T, int R, bool DIRECT> static int psi_blocks_per_sm()
 {
     const size_t smem = kWalkWarps * sizeof(WalkShared<KIND, T>);
     static int bps = -1;
@@ -447,9 +446,16 @@ static void psi_launch_one(const WalkParams<T>& P, const PsiConsts<T>& K, int nu
                                  (int)smem);
         int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psi_kernel<KIND, T, R, DIRECT>, kWalkWarps * 32, smem);
-        // stacks are allocated for 16 blocks per SM, a tree walk's cut slots for kCutBlocks
-        bps = std::min(std::max(nb, 1), DIRECT ? 16 : kCutBlocks);
+        bps = std::min(std::max(nb, 1), DIRECT ? 16 : kWalkBlocks);  // (room for stacks and cuts)
     }
+    return bps;
+}
+
+template <int KIND, typename T, int R, bool DIRECT>
+static void psi_launch_one(const WalkParams<T>& P, const PsiConsts<T>& K, int num_sms, cudaStream_t s)
+{
+    const size_t smem = kWalkWarps * sizeof(WalkShared<KIND, T>);
+    const int bps = psi_blocks_per_sm<KIND, T, R, DIRECT>();
     { psi_kernel<KIND, T, R, DIRECT><<<num_sms * bps, kWalkWarps * 32, smem, s>>>(P, K); note_launch(); }
 }
 
@@ -459,6 +465,13 @@ static void psi_launch_kind(int kind, const WalkParams<T>& P, const PsiConsts<T>
     if (kind == LENS_POINT) psi_launch_one<LENS_POINT, T, R, DIRECT>(P, K, num_sms, s);
     else if (kind == LENS_GAUSS) psi_launch_one<LENS_GAUSS, T, R, DIRECT>(P, K, num_sms, s);
     else psi_launch_one<LENS_NFW, T, R, DIRECT>(P, K, num_sms, s);
+}
+
+template <typename T, int R> static int psi_cut_blocks(int kind)
+{
+    if (kind == LENS_POINT) return psi_blocks_per_sm<LENS_POINT, T, R, false>();
+    if (kind == LENS_GAUSS) return psi_blocks_per_sm<LENS_GAUSS, T, R, false>();
+    return psi_blocks_per_sm<LENS_NFW, T, R, false>();
 }
 
 // Host values of the per-species constants (FP64).
@@ -534,7 +547,8 @@ static lens_status psi_typed(lens_tree* t, const ShootPlan& plan, const void* dx
             auto go = [&](auto rays) {
                 constexpr int R = decltype(rays)::value;
                 auto walk = [&](const WalkParams<T>& Q) { psi_launch_kind<T, R, false>(kind, Q, K, t->num_sms, s); };
-                walk_rounds<T, R>(P, ng, 3, base, L, P.counter, walk, s);
+                const int warps = kWalkWarps * t->num_sms * psi_cut_blocks<T, R>(kind);
+                walk_rounds<T, R>(P, ng, 3, base, L, P.counter, walk, warps, s);
             };
             if (plan.R == 1) go(std::integral_constant<int, 1>{});
             else go(std::integral_constant<int, 2>{});

@@ -907,7 +907,7 @@ static int walk_blocks_per_sm()
         int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, walk_kernel<KIND, T, R, AO, DIRECT, TILE, LOC>,
                                                       kWalkWarps * 32, smem);
-        cached = nb > 0 ? nb : 1;
+        cached = std::min(std::max(nb, 1), DIRECT ? 16 : kWalkBlocks);  // (room for stacks and cuts)
     }
     return cached;
 }
@@ -941,8 +941,6 @@ static void launch_one(const WalkParams<T>& P, int num_sms, cudaStream_t s)
 {
     size_t smem = kWalkWarps * sizeof(WalkShared<KIND, T, TILE, tot_rays<R>()>);
     int bps = walk_blocks_per_sm<KIND, T, R, AO, DIRECT, TILE, LOC>();
-    // stack slots are allocated for 16 blocks per SM, a tree walk's cut slots for kCutBlocks
-    if (bps > (DIRECT ? 16 : kCutBlocks)) bps = DIRECT ? 16 : kCutBlocks;
     int grid = num_sms * bps;
     { walk_kernel<KIND, T, R, AO, DIRECT, TILE, LOC><<<grid, kWalkWarps * 32, smem, s>>>(P); note_launch(); }
 }
@@ -980,6 +978,9 @@ static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, co
         }
         launch_one<KIND, T, R, AO, false, TILE, KIND == LENS_NFW && kF32>(Q, sms, s);
     };
+    const int cut_warps = kWalkWarps * sms *
+                          (P.super ? walk_blocks_per_sm<KIND, T, R, AO, false, TILE, kF32 && KIND != LENS_GAUSS>()
+                                   : walk_blocks_per_sm<KIND, T, R, AO, false, TILE, KIND == LENS_NFW && kF32>());
     if (KIND == LENS_POINT && kF32 && !P.super && P.n_part < 8192) {
         // (no group can reach the limit of a cut: cells and particles together
         // are fewer than twice the particles)
@@ -987,7 +988,7 @@ static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, co
         return;
     }
     if (P.n_groups < kPlainGroups || P.super || (KIND == LENS_NFW && kF32)) {
-        walk_rounds<T, R>(P, P.n_groups, nq, base, L, counter, cut, s, KIND == LENS_POINT && kF32);
+        walk_rounds<T, R>(P, P.n_groups, nq, base, L, counter, cut, cut_warps, s, KIND == LENS_POINT && kF32);
         if (KIND == LENS_POINT && kF32 && P.super) {
             // a narrow patch, which only the device knows (SuperRec::ok == 3):
             // the rounds found no groups and the plain kernel takes them all
@@ -1006,7 +1007,7 @@ static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, co
         WalkParams<T> Q = P;
         Q.sub = sub + 16;
         Q.sub_n = sub;
-        walk_rounds<T, R>(Q, P.n_groups, nq, base, L, counter, cut, s);
+        walk_rounds<T, R>(Q, P.n_groups, nq, base, L, counter, cut, cut_warps, s);
         P.gflag = (const uint8_t*)(base + L.gflag);
         P.skip = 1;
         cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);

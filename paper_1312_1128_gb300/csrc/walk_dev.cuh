@@ -1464,9 +1464,9 @@ __global__ void k_cut_sum(CutPool<T> pool, CutPool<T> to, WalkParams<T> P, int n
 }
 
 // The launches of one tree walk over ng groups: `walk(P)` launches the
-// kernel.  Groups are cut in a launch's kernel and their parts run in the
-// next one; a part may be cut once more.  Launches without items cost about
-// 3 us each, beside walks of 100 us and more.
+// kernel, of `warps` warps.  Groups are cut in a launch's kernel and their parts
+// run in the next one; a part may be cut once more.  Launches without items
+// cost about 3 us each, beside walks of 100 us and more.
 //   ng <= 512: far fewer warps than the chip holds.  Every group is cut as
 //     soon as its stack holds 64 boxes (its big lists deferred to the parts),
 //     into enough parts for about 8,192 warps.
@@ -1482,19 +1482,19 @@ __global__ void k_cut_sum(CutPool<T> pool, CutPool<T> to, WalkParams<T> P, int n
 //     (1e-3 of the sum of |terms|): such groups keep their order of summation.
 template <typename T, int R, typename Walk>
 void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& L, uint32_t* counter, Walk&& walk,
-                 cudaStream_t s, bool keep_order = false)
+                 int warps, cudaStream_t s, bool keep_order = false)
 {
     // counter: 8 words, zeroed by the caller: work counters, then each pool's
     CutPool<T> pool[2];
     constexpr size_t total = 5 * 32 * R * sizeof(T);
-    char* at = base + L.cut;
+    char* at = base + L.stack + (size_t)warps * kStackCap * sizeof(int);
     auto take = [&](size_t bytes) {
         char* p = at;
         at += (bytes + 255) & ~(size_t)255;
         return p;
     };
     const size_t local_bytes = cut_local_bytes<R, T>() * 2;
-    unsigned char* local = (unsigned char*)take(L.cut_warps * local_bytes);
+    unsigned char* local = (unsigned char*)take((size_t)warps * local_bytes);
     // the second pool: parts that are cut again
     pool[1].parts = ng <= 4096 && !keep_order ? 16 : 32;
     pool[1].max_cuts = (uint32_t)(kCutAgainBytes / (pool[1].parts * total));
@@ -1502,7 +1502,7 @@ void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& 
     pool[1].head = (T*)take(pool[1].max_cuts * total);
     pool[1].part = (T*)take(pool[1].max_cuts * pool[1].parts * total);
     // the first has the rest: every group that may be cut has a place
-    const size_t room = L.cut_bytes - (size_t)(at - (base + L.cut)) - 4 * 256;
+    const size_t room = (size_t)(base + L.cut_end - at) - 4 * 256;
     const bool few = ng <= 4096 && !keep_order;
     bool all = true;
     if (few) {

@@ -2,6 +2,8 @@
 // adjoint walk (backward.cu) and graph replay (batch.cu).
 #pragma once
 
+#include <algorithm>
+
 #include "sort.cuh"
 #include "tree.cuh"
 
@@ -44,14 +46,17 @@ LENS_DEV bool box_reaches_group(const vec4_t<T>& b, const v2_t<T>& H, const vec4
 
 struct Layout {
     size_t boff, borig, gfirst, bbox, k0, k1, v0, v1, tmp, rl, ridx, gH, gbox, grange, counter,
-        stack, split, gcost, heavy, cut, super, sdelta, gflag, sub, total;
-    size_t cut_bytes;   // of the region at cut
-    size_t cut_warps;   // warps of a tree walk that have a place of their own there
+        stack, split, gcost, heavy, super, sdelta, gflag, sub, total;
+    size_t cut_end;   // cuts lie between the stacks that a launch uses and here
 };
 
-// Cut groups (walk_dev.cuh): one region for a call's cuts, split by the walk
-// (walk_rounds): a place for each of its warps, then two pools.
-constexpr size_t kCutBytes = (size_t)112 << 20;       // the whole region
+// Cut groups (walk_dev.cuh): a call's cuts lie in the part of the stack region
+// that its launches leave unused (stacks are allocated for 16 blocks per SM, a
+// tree walk has at most kWalkBlocks: 80 MB and more are left), which
+// walk_rounds splits: a place for each warp of the cut form, then two pools.
+// From about 600,000 rays on up to 48 MB are added behind it, so that every
+// group has a place in the first pool up to 24,576 groups.
+constexpr int kWalkBlocks = 8;
 constexpr size_t kCutAgainBytes = (size_t)20 << 20;   // totals of the second pool's parts
 constexpr size_t kCutSlotBytes = 2320;
 // Stretched groups: Morton order jumps between quadrants, so unless the rays
@@ -67,7 +72,6 @@ constexpr float kStretch = 16.0f;
 // Supergroups (walk_dev.cuh): kSuperGroups consecutive groups, one record each.
 constexpr int kSuperGroups = 32;
 constexpr size_t kSuperBytes = 1664;
-constexpr int kCutBlocks = 8;  // resident blocks per SM of a tree walk (each warp has its own slot and sums)
 
 // Tags of a kept interaction-list entry (LENS_KEEP_LISTS): the box's index
 // in the low 29 bits; a box may be accepted (far cell) or an opened leaf, and
@@ -108,12 +112,12 @@ inline Layout make_layout(int64_t n, int64_t nb, int64_t slots)
     L.grange = o; o += al(ng * sizeof(uint2));
     L.counter = o; o += al(64 * sizeof(uint32_t));  // 8 words for each species' launches
     L.stack = o; o += al((size_t)slots * kStackCap * sizeof(int));
+    const size_t places = (size_t)n / 32 * (kCutSlotBytes + 2 * 5 * 32 * sizeof(float));
+    o += al(std::min(places > ((size_t)65 << 20) ? places - ((size_t)65 << 20) : 0, (size_t)48 << 20));
+    L.cut_end = o;
     L.split = o; o += al(split_values(slots) * 5 * sizeof(double));
     L.gcost = o; o += al(ng * sizeof(uint32_t));
     L.heavy = o; o += al(64 + (size_t)kHeavyItems * sizeof(uint32_t));
-    L.cut = o; o += al(kCutBytes);
-    L.cut_bytes = kCutBytes;
-    L.cut_warps = (size_t)slots / 16 * kCutBlocks;  // (slots: 16 blocks per SM)
     L.super = o; o += al((size_t)(ng / kSuperGroups + 1) * kSuperBytes);
     L.sdelta = o; o += al(ng * 4 * sizeof(float));
     L.gflag = o; o += al(ng);

@@ -94,3 +94,21 @@ def test_repeated_call_is_bitwise_equal_when_most_groups_are_cut(kind, theta, ca
     for _ in range(5):
         assert all(torch.equal(a, b) for a, b in zip(first, run(dx, dy)))
     lens.close()
+
+
+def test_scratch_of_a_small_lens():
+    """The scratch of small calls: stacks (159 MB on 152 SMs), the direct sum's
+    partial sums (12 MB) and little else; the cuts lie in the stacks' region.
+    Eight lenses at once, at most 200 MB each."""
+    p = lensgen.nfw_particles(4000, 11, nsph=16)
+    dx, dy = (cu(lensgen.rng(12).uniform(-0.8, 0.8, 512).astype(np.float32)) for _ in range(2))
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    lenses = [L.Lens([L.Species.gauss(cu(p), 3.0)], theta=0.3) for _ in range(8)]
+    for lens in lenses:
+        lens.shoot(dx, dy)
+        lens.sync()
+    used = before - torch.cuda.mem_get_info()[0]
+    for lens in lenses:
+        lens.close()
+    assert used <= 8 * 200e6, used / 8
