@@ -64,11 +64,13 @@ LENS_DEV float2 ein_poly2(float2 u)
     return __fmul2_rn(ein_cheb2<8>(t, make_float2(top, top)), u);
 }
 
-template <int KIND, typename T, int R> struct PsiCtx {
+// DEFER: the cut form, which puts long lists aside; otherwise a whole group's walk,
+// or a direct sum.
+template <int KIND, typename T, int R, bool DEFER> struct PsiCtx {
     using value_type = T;
     using Buf = WalkBuf<KIND, T>;
     static constexpr int kKind = KIND, kR = R;
-    static constexpr bool kCuts = true;
+    static constexpr bool kCuts = true, kDefer = DEFER;
     static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
     const WalkParams<T>& P;
     const PsiConsts<T> K;
@@ -87,7 +89,7 @@ template <int KIND, typename T, int R> struct PsiCtx {
     T part[R][3];              // psi, alpha1, alpha2 of the current flush
     T tot_s[R][3], tot_c[R][3];  // compensated totals
 
-    LENS_DEV PsiCtx(const WalkParams<T>& p, const PsiConsts<T>& k, WalkShared<KIND, T>& s)
+    template <class S> LENS_DEV PsiCtx(const WalkParams<T>& p, const PsiConsts<T>& k, S& s)
         : P(p), K(k), B(&s.buf), Rg(&s.rng), Cut(&s.cut) {}
 
     LENS_DEV void zero()
@@ -345,45 +347,47 @@ template <int KIND, typename T, int R> struct PsiCtx {
     }
 };
 
-template <int KIND, typename T, int R, bool DIRECT>
-__global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, PsiConsts<T> K)
+// FORM 0: the direct sum; 1: a tree walk of whole groups (a heavy one hands the
+// rest of its walk to parts); 2: the cut form, for parts and for calls whose
+// groups are all cut (walk_rounds).
+template <int KIND, typename T, int FORM>
+using PsiShared = std::conditional_t<FORM == 2, WalkShared<KIND, T>, PlainShared<KIND, T>>;
+
+template <int KIND, typename T, int R, int FORM>
+__global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(const __grid_constant__ WalkParams<T> P,
+                                                              const __grid_constant__ PsiConsts<T> K)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr bool DIRECT = FORM == 0;
     const unsigned full = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WalkShared<KIND, T>& S = reinterpret_cast<WalkShared<KIND, T>*>(smem_raw)[warp];
+    PsiShared<KIND, T, FORM>& S = reinterpret_cast<PsiShared<KIND, T, FORM>*>(smem_raw)[warp];
     int* stack = P.stack + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
-    PsiCtx<KIND, T, R> C(P, K, S);
-    uint32_t ridx[R];
-    bool rv[R];
+    PsiCtx<KIND, T, R, FORM == 2> C(P, K, S);
     for (;;) {
         uint32_t g = 0;
-        if constexpr (DIRECT) {
+        if constexpr (FORM == 2) {
+            if (!next_item<R>(P, stack, S.cut)) break;
+            g = S.cut.g;
+        } else {
             if (lane == 0) g = atomicAdd(P.counter, 1u);
             g = __shfl_sync(full, g, 0);
             if ((int64_t)g >= P.n_groups) break;
-        } else {
-            if (!next_item<R>(P, stack, S.cut)) break;
-            g = S.cut.g;
         }
-        const bool head = DIRECT || S.cut.item == kNoItem;  // the group's first (or only) item
+        const bool head = FORM != 2 || S.cut.item == kNoItem;  // the group's first (or only) item
+        if constexpr (FORM == 1) whole_group(P, S.cut, g, stack);
         C.H = P.gH[g];
         C.box = P.gbox[g];
-        const uint2 rg = P.grange[g];
+        const uint2 first = P.grange[g];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int k = r * 32 + lane;
-            rv[r] = k < (int)rg.y;
-            if (rv[r]) {
-                const v2_t<T> l = P.ray_l[rg.x + k];
-                C.lx[r] = l.x;
-                C.ly[r] = l.y;
-                ridx[r] = P.ray_idx[rg.x + k];
-            } else {
-                C.lx[r] = C.box.x;
-                C.ly[r] = C.box.y;
-                ridx[r] = 0;
-            }
+            v2_t<T> l;
+            l.x = C.box.x;
+            l.y = C.box.y;
+            if (k < (int)first.y) l = P.ray_l[first.x + k];
+            C.lx[r] = l.x;
+            C.ly[r] = l.y;
         }
         C.nf = C.nn = C.nb = 0;
         C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
@@ -398,6 +402,14 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
                 C.flush_near();
             }
             if (P.n_halos > 0) C.halos();
+        } else if constexpr (FORM == 1) {
+            C.zero();
+            traverse(C, stack, 1);
+            C.flush_far();
+            C.flush_near();
+            C.flush_big();
+            if (P.n_halos > 0) C.halos();
+            if (S.cut.sp > 0) cut_now<R, false>(P.cut, S.cut, stack, S.cut.sp);
         } else {
             do {  // (once, or once for each part of a cut whose pool was full)
                 C.zero();
@@ -413,16 +425,21 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
                          return C.tot_s[r][q] + C.tot_c[r][q]; }));
         }
         __syncwarp();
-        if constexpr (DIRECT) count_item(C, g, rg.y, head);
+        // (read again: kept in registers over the walk they cost it spills)
+        if constexpr (!DIRECT) g = S.cut.g;
+        const uint2 rg = P.grange[g];
+        if constexpr (FORM != 2) count_item(C, g, rg.y, head);
         T* tot = DIRECT ? nullptr : item_totals<R>(P.cut, S.cut);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            if (!rv[r] && !tot) continue;
-            const uint32_t i = ridx[r];
+            const int k = r * 32 + lane;
+            const bool ray = k < (int)rg.y;
+            if (!ray && !tot) continue;
+            const uint32_t i = ray ? P.ray_idx[rg.x + k] : 0u;
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 T val = C.tot_s[r][q] + C.tot_c[r][q];
-                if (!DIRECT && S.cut.local) val = local_total<R>(P.cut, r, q);
+                if (FORM == 2 && S.cut.local) val = local_total<R>(P.cut, r, q);
                 if (tot) {
                     tot[(q * R + r) * 32 + lane] = val;
                     continue;
@@ -436,42 +453,43 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(WalkParams<T> P, P
     }
 }
 
-template <int KIND, typename T, int R, bool DIRECT> static int psi_blocks_per_sm()
+template <int KIND, typename T, int R, int FORM> static int psi_blocks_per_sm()
 {
-    const size_t smem = kWalkWarps * sizeof(WalkShared<KIND, T>);
+    const size_t smem = kWalkWarps * sizeof(PsiShared<KIND, T, FORM>);
     static int bps = -1;
     if (bps < 0) {
         if (smem > 48 * 1024)
-            cudaFuncSetAttribute(psi_kernel<KIND, T, R, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(psi_kernel<KIND, T, R, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem);
         int nb = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psi_kernel<KIND, T, R, DIRECT>, kWalkWarps * 32, smem);
-        bps = std::min(std::max(nb, 1), DIRECT ? 16 : kWalkBlocks);  // (room for stacks and cuts)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psi_kernel<KIND, T, R, FORM>, kWalkWarps * 32, smem);
+        bps = std::min(std::max(nb, 1), FORM == 0 ? 16 : kWalkBlocks);  // (room for stacks and cuts)
     }
     return bps;
 }
 
-template <int KIND, typename T, int R, bool DIRECT>
+template <int KIND, typename T, int R, int FORM>
 static void psi_launch_one(const WalkParams<T>& P, const PsiConsts<T>& K, int num_sms, cudaStream_t s)
 {
-    const size_t smem = kWalkWarps * sizeof(WalkShared<KIND, T>);
-    const int bps = psi_blocks_per_sm<KIND, T, R, DIRECT>();
-    { psi_kernel<KIND, T, R, DIRECT><<<num_sms * bps, kWalkWarps * 32, smem, s>>>(P, K); note_launch(); }
+    const size_t smem = kWalkWarps * sizeof(PsiShared<KIND, T, FORM>);
+    const int bps = psi_blocks_per_sm<KIND, T, R, FORM>();
+    { psi_kernel<KIND, T, R, FORM><<<num_sms * bps, kWalkWarps * 32, smem, s>>>(P, K); note_launch(); }
 }
 
-template <typename T, int R, bool DIRECT>
+template <typename T, int R, int FORM>
 static void psi_launch_kind(int kind, const WalkParams<T>& P, const PsiConsts<T>& K, int num_sms, cudaStream_t s)
 {
-    if (kind == LENS_POINT) psi_launch_one<LENS_POINT, T, R, DIRECT>(P, K, num_sms, s);
-    else if (kind == LENS_GAUSS) psi_launch_one<LENS_GAUSS, T, R, DIRECT>(P, K, num_sms, s);
-    else psi_launch_one<LENS_NFW, T, R, DIRECT>(P, K, num_sms, s);
+    if (kind == LENS_POINT) psi_launch_one<LENS_POINT, T, R, FORM>(P, K, num_sms, s);
+    else if (kind == LENS_GAUSS) psi_launch_one<LENS_GAUSS, T, R, FORM>(P, K, num_sms, s);
+    else psi_launch_one<LENS_NFW, T, R, FORM>(P, K, num_sms, s);
 }
 
-template <typename T, int R> static int psi_cut_blocks(int kind)
+template <typename T, int R, int FORM> static int psi_warps(int kind, int num_sms)
 {
-    if (kind == LENS_POINT) return psi_blocks_per_sm<LENS_POINT, T, R, false>();
-    if (kind == LENS_GAUSS) return psi_blocks_per_sm<LENS_GAUSS, T, R, false>();
-    return psi_blocks_per_sm<LENS_NFW, T, R, false>();
+    const int b = kind == LENS_POINT   ? psi_blocks_per_sm<LENS_POINT, T, R, FORM>()
+                  : kind == LENS_GAUSS ? psi_blocks_per_sm<LENS_GAUSS, T, R, FORM>()
+                                       : psi_blocks_per_sm<LENS_NFW, T, R, FORM>();
+    return kWalkWarps * num_sms * b;
 }
 
 // Host values of the per-species constants (FP64).
@@ -525,6 +543,7 @@ static lens_status psi_typed(lens_tree* t, const ShootPlan& plan, const void* dx
     P.ray_l = (T2*)(base + L.rl);
     P.ray_idx = (uint32_t*)(base + L.ridx);
     P.n_groups = (int64_t)plan.ng;
+    P.n_rays = plan.n;
     P.stack = (int*)(base + L.stack);
     P.err = t->d_err;
     P.stats = (flags & LENS_COUNT) ? t->d_stats : nullptr;
@@ -541,14 +560,23 @@ static lens_status psi_typed(lens_tree* t, const ShootPlan& plan, const void* dx
         const int64_t ng = (int64_t)plan.ng;
         // (a lens without particles has nothing to walk: the direct form)
         if (direct || P.n_part == 0) {
-            if (plan.R == 1) psi_launch_kind<T, 1, true>(kind, P, K, t->num_sms, s);
-            else psi_launch_kind<T, 2, true>(kind, P, K, t->num_sms, s);
+            if (plan.R == 1) psi_launch_kind<T, 1, 0>(kind, P, K, t->num_sms, s);
+            else psi_launch_kind<T, 2, 0>(kind, P, K, t->num_sms, s);
         } else {
             auto go = [&](auto rays) {
                 constexpr int R = decltype(rays)::value;
-                auto walk = [&](const WalkParams<T>& Q) { psi_launch_kind<T, R, false>(kind, Q, K, t->num_sms, s); };
-                const int warps = kWalkWarps * t->num_sms * psi_cut_blocks<T, R>(kind);
-                walk_rounds<T, R>(P, ng, 3, base, L, P.counter, walk, warps, s);
+                auto cut = [&](const WalkParams<T>& Q) { psi_launch_kind<T, R, 2>(kind, Q, K, t->num_sms, s); };
+                auto whole = [&](const WalkParams<T>& Q) { psi_launch_kind<T, R, 1>(kind, Q, K, t->num_sms, s); };
+                // few groups, and mid-sized calls of larger trees: the cut
+                // form; otherwise whole groups, whose kernel has 16 to 24
+                // registers less (20,000 particles: 1.04 to 1.2 times as fast)
+                const CutPlan cp{ng <= kFewGroups, false, false};
+                const int cut_warps = psi_warps<T, R, 2>(kind, t->num_sms);
+                const int warps = std::max(cut_warps, psi_warps<T, R, 1>(kind, t->num_sms));
+                const bool cuts = cp.few || (ng < 24576 && P.n_part >= 24576) || !cuts_fit<T, R>(ng, L, warps, cut_warps);
+                if (never_cut(t, ng, P.n_rays, P.n_part, cp)) whole(P);
+                else if (cuts) walk_rounds<T, R>(P, cp, 3, base, L, P.counter, cut, cut, cut_warps, cut_warps, s);
+                else walk_rounds<T, R>(P, cp, 3, base, L, P.counter, whole, cut, warps, cut_warps, s);
             };
             if (plan.R == 1) go(std::integral_constant<int, 1>{});
             else go(std::integral_constant<int, 2>{});

@@ -474,8 +474,11 @@ walk_kernel(const __grid_constant__ WalkParams<T> P)
     }
 }
 
-// The plain tree walk: whole groups, with P.skip all but the stretched ones.
-template <int KIND, typename T, int R, bool AO, int TILE>
+// The plain tree walk: whole groups, without expansions, fewer registers than
+// the cut form; with P.skip all but the stretched ones.  CUTS: heavy groups
+// (cut_limit) hand the rest of their walk to parts (FP32 point masses only: the
+// code cost Gaussian trees 4 to 8 % on calls that cut nothing).
+template <int KIND, typename T, int R, bool AO, int TILE, bool CUTS>
 __global__ void __launch_bounds__(kWalkWarps * 32, sizeof(T) == 4 ? (R == 4 ? 4 : (R == 2 ? 5 : 6)) : 2)
 walk_plain(const __grid_constant__ WalkParams<T> P)
 {
@@ -484,34 +487,28 @@ walk_plain(const __grid_constant__ WalkParams<T> P)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     PlainShared<KIND, T, TILE, tot_rays<R>()>& S = reinterpret_cast<PlainShared<KIND, T, TILE, tot_rays<R>()>*>(smem_raw)[warp];
     int* stack = P.stack + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
-    PlainCtx<KIND, T, R, AO, TILE> C(P, &S.buf, &S.tot, &S.rng);
+    PlainCtx<KIND, T, R, AO, TILE, CUTS> C(P, &S.buf, &S.tot, &S.rng, &S.cut);
     if (P.super && P.super[0].ok != 3) return;  // the supergroups' walk has run
-    uint32_t ridx[R];
-    bool rv[R];
     for (;;) {
         uint32_t item = 0;
         if (lane == 0) item = atomicAdd(P.counter, 1u);
         item = __shfl_sync(full, item, 0);
         if ((int64_t)item >= P.n_groups) break;
         const uint32_t g = P.order ? P.order[item] : item;
-        if (P.skip && P.gflag[g]) continue;
+        if (!CUTS && P.skip && P.gflag[g]) continue;
+        whole_group(P, S.cut, g, stack);
         C.H = P.gH[g];
         C.box = P.gbox[g];
-        const uint2 rg = P.grange[g];
+        const uint2 first = P.grange[g];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int k = r * 32 + lane;
-            rv[r] = k < (int)rg.y;
-            if (rv[r]) {
-                const v2_t<T> l = P.ray_l[rg.x + k];
-                C.lx[r] = l.x;
-                C.ly[r] = l.y;
-                ridx[r] = P.ray_idx[rg.x + k];
-            } else {
-                C.lx[r] = C.box.x;
-                C.ly[r] = C.box.y;
-                ridx[r] = 0;
-            }
+            v2_t<T> l;
+            l.x = C.box.x;
+            l.y = C.box.y;
+            if (k < (int)first.y) l = P.ray_l[first.x + k];
+            C.lx[r] = l.x;
+            C.ly[r] = l.y;
             C.part[r].zero();
         }
         C.tot_zero();
@@ -520,24 +517,33 @@ walk_plain(const __grid_constant__ WalkParams<T> P)
         C.rec = P.list_ids ? P.list_ids + (int64_t)g * P.list_K : nullptr;
         C.rec_n = 0;
         C.rec_cap = P.list_K;
-        if (lane == 0) stack[0] = 0;
-        __syncwarp();
         const bool whole = traverse(C, stack, 1);
         if (C.rec && lane == 0)
-            P.list_n[g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListTooLong;
+            P.list_n[S.cut.g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListTooLong;
         C.flush_far();
         C.flush_near();
         if constexpr (KIND != LENS_POINT) C.flush_big();
         if (P.n_halos > 0) C.halos(P.halos, P.n_halos);
-        count_item(C, g, rg.y, true);
+        // (read again: kept in registers over the walk they cost it spills)
+        const uint2 rg = P.grange[S.cut.g];
+        count_item(C, S.cut.g, rg.y, true);
+        if (CUTS && S.cut.sp > 0) cut_now<R, false>(P.cut, S.cut, stack, S.cut.sp);
+        __syncwarp();
+        T* tot = CUTS ? item_totals<R>(P.cut, S.cut) : nullptr;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            if (!rv[r]) continue;
-            const uint32_t i = ridx[r];
+            const int k = r * 32 + lane;
+            const bool ray = k < (int)rg.y;
+            if (!ray && !tot) continue;
+            const uint32_t i = ray ? P.ray_idx[rg.x + k] : 0u;
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
                 if (AO && q >= 2) break;
                 T val = C.tot_get(r, q);
+                if (tot) {
+                    tot[(q * R + r) * 32 + lane] = val;
+                    continue;
+                }
                 if (P.accumulate) val += P.out[q][i];
                 P.out[q][i] = val;
             }
@@ -546,19 +552,27 @@ walk_plain(const __grid_constant__ WalkParams<T> P)
     }
 }
 
-template <int KIND, typename T, int R, bool AO, int TILE>
+template <int KIND, typename T, int R, bool AO, int TILE, bool CUTS> static int plain_blocks_per_sm()
+{
+    constexpr size_t smem = kWalkWarps * sizeof(PlainShared<KIND, T, TILE, tot_rays<R>()>);
+    constexpr auto kernel = walk_plain<KIND, T, R, AO, TILE, CUTS>;
+    static const int bps = [] {
+        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        int nb = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kWalkWarps * 32, smem);
+        // (stacks are allocated for 16 blocks per SM; where cuts lie behind them: kWalkBlocks)
+        return std::min(std::max(nb, 1), CUTS ? kWalkBlocks : 16);
+    }();
+    return bps;
+}
+
+template <int KIND, typename T, int R, bool AO, int TILE, bool CUTS = false>
 static void launch_plain(const WalkParams<T>& P, int num_sms, cudaStream_t s)
 {
     constexpr size_t smem = kWalkWarps * sizeof(PlainShared<KIND, T, TILE, tot_rays<R>()>);
-    static const int bps = [] {
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(walk_plain<KIND, T, R, AO, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(walk_plain<KIND, T, R, AO, TILE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        int nb = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, walk_plain<KIND, T, R, AO, TILE>, kWalkWarps * 32, smem);
-        return std::min(std::max(nb, 1), 16);  // stack slots are allocated for 16 blocks per SM
-    }();
-    walk_plain<KIND, T, R, AO, TILE><<<num_sms * bps, kWalkWarps * 32, smem, s>>>(P);
+    const int bps = plain_blocks_per_sm<KIND, T, R, AO, TILE, CUTS>();
+    walk_plain<KIND, T, R, AO, TILE, CUTS><<<num_sms * bps, kWalkWarps * 32, smem, s>>>(P);
     note_launch();
 }
 
@@ -960,60 +974,89 @@ static void launch_direct(int kind, bool ao, const WalkParams<T>& P, int num_sms
     else launch_kind<T, R, false>(kind, P, num_sms, s);
 }
 
-// The one-warp tree walk of all groups: in rounds of cut groups, or, from
-// kPlainGroups groups on and without expansions, the stretched groups so and
-// the others by the plain kernel (the cut form's registers cost it 5 %).
+// The one-warp tree walk of all groups.
+//   FP32 NFW trees (expansions) and, up to 4,096 groups, all but FP32 point
+//     masses: the cut form.
+//   FP32 point masses: the plain kernel with cuts (up to 1,024 groups the cut
+//     form: every warp counts there, and its steps are shorter: 504 groups of
+//     67,587 stars 1.11 ms, 1.22).  With supergroups the cut form with
+//     expansions or, as only the device knows, the plain kernel: the other of
+//     the two launches finds no work.
+//   The others: from kPlainGroups groups on the stretched groups by the cut
+//     form and the rest by the plain kernel, whose 80 to 96 registers the cut
+//     form's 96 to 128 cost 5 to 10 %; below, all by the cut form, which cuts
+//     heavy groups too (1e5 and 1e6 particles, 4,300 to 22,000 groups: 1.3 to 5
+//     times as fast as the plain kernel), unless the tree has fewer than
+//     kPlainParticles (20,000: no group is heavy, 1.03 to 1.08).
+constexpr int64_t kPlainGroups = 24576, kPlainParticles = 24576;
 template <int KIND, typename T, int R, bool AO, int TILE>
 static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, const Layout& L, cudaStream_t s)
 {
-    constexpr bool kF32 = sizeof(T) == 4;
+    constexpr bool kF32 = sizeof(T) == 4, kNfw = KIND == LENS_NFW && kF32, kPoint = KIND == LENS_POINT && kF32;
     const int sms = t->num_sms;
+    const int64_t ng = P.n_groups;
     uint32_t* counter = P.counter;
     auto cut = [&](const WalkParams<T>& Q) {
-        if constexpr (KIND == LENS_POINT && kF32) {
+        if constexpr (kPoint) {
             if (Q.super) {
                 launch_one<KIND, T, R, AO, false, TILE, true>(Q, sms, s);
                 return;
             }
         }
-        launch_one<KIND, T, R, AO, false, TILE, KIND == LENS_NFW && kF32>(Q, sms, s);
+        launch_one<KIND, T, R, AO, false, TILE, kNfw>(Q, sms, s);
     };
-    const int cut_warps = kWalkWarps * sms *
-                          (P.super ? walk_blocks_per_sm<KIND, T, R, AO, false, TILE, kF32 && KIND != LENS_GAUSS>()
-                                   : walk_blocks_per_sm<KIND, T, R, AO, false, TILE, KIND == LENS_NFW && kF32>());
-    if (KIND == LENS_POINT && kF32 && !P.super && P.n_part < 8192) {
-        // (no group can reach the limit of a cut: cells and particles together
-        // are fewer than twice the particles)
-        launch_plain<KIND, T, R, AO, TILE>(P, sms, s);
-        return;
-    }
-    if (P.n_groups < kPlainGroups || P.super || (KIND == LENS_NFW && kF32)) {
-        walk_rounds<T, R>(P, P.n_groups, nq, base, L, counter, cut, cut_warps, s, KIND == LENS_POINT && kF32);
-        if (KIND == LENS_POINT && kF32 && P.super) {
-            // a narrow patch, which only the device knows (SuperRec::ok == 3):
-            // the rounds found no groups and the plain kernel takes them all
-            // (131,772 stars, 1527^2 rays over 4.6e-5: 3.8 ms, 4.9 ms in the
-            // rounds); otherwise its blocks return at once
+    const int cut_warps = kWalkWarps * sms * (P.super ? walk_blocks_per_sm<KIND, T, R, AO, false, TILE, kPoint || kNfw>()
+                                                      : walk_blocks_per_sm<KIND, T, R, AO, false, TILE, kNfw>());
+    const CutPlan plan{ng <= kFewGroups && !kPoint, kPoint, false};
+    if constexpr (kNfw) {
+        if (never_cut(t, ng, P.n_rays, P.n_part, plan)) cut(P);
+        else walk_rounds<T, R>(P, plan, nq, base, L, counter, cut, cut, cut_warps, cut_warps, s);
+    } else if constexpr (kPoint) {
+        const int warps = std::max(cut_warps, kWalkWarps * sms * plain_blocks_per_sm<KIND, T, R, AO, TILE, true>());
+        const bool fit = cuts_fit<T, R>(ng, L, warps, cut_warps);
+        auto groups = [&](const WalkParams<T>& Q) {
+            const bool whole = fit && ng > 1024;
+            if (Q.super || !whole) cut(Q);
+            if (!Q.super && !whole) return;
+            WalkParams<T> W = Q;
+            if (Q.super) W.counter = counter + 6;
+            if (fit) launch_plain<KIND, T, R, AO, TILE, true>(W, sms, s);
+            else launch_plain<KIND, T, R, AO, TILE>(W, sms, s);
+        };
+        if (never_cut(t, ng, P.n_rays, P.n_part, plan)) {
+            WalkParams<T> W = P;
+            if (P.super) {
+                cut(P);
+                W.counter = counter + 6;
+            }
+            launch_plain<KIND, T, R, AO, TILE>(W, sms, s);
+        } else {
+            walk_rounds<T, R>(P, plan, nq, base, L, counter, groups, cut, warps, cut_warps, s);
+        }
+    } else {
+        if (plan.few && never_cut(t, ng, P.n_rays, P.n_part, plan)) {
+            launch_plain<KIND, T, R, AO, TILE>(P, sms, s);
+            return;
+        }
+        if (plan.few || (ng < kPlainGroups && !(kF32 && P.n_part < kPlainParticles))) {
+            walk_rounds<T, R>(P, plan, nq, base, L, counter, cut, cut, cut_warps, cut_warps, s);
+            return;
+        }
+        if (P.n_part > 4 * ng) {
+            // (fewer particles: even a group that meets all of them is done
+            // before the others; lens fit, 1e5 particles, 31,250 groups)
+            const uint32_t* sub = (const uint32_t*)(base + L.sub);
+            WalkParams<T> Q = P;
+            Q.sub = sub + 16;
+            Q.sub_n = sub;
+            walk_rounds<T, R>(Q, CutPlan{false, false, true}, nq, base, L, counter, cut, cut, cut_warps, cut_warps, s);
+            P.gflag = (const uint8_t*)(base + L.gflag);
+            P.skip = 1;
             cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
             P.counter = counter;
-            launch_plain<KIND, T, R, AO, TILE>(P, sms, s);
         }
-        return;
+        launch_plain<KIND, T, R, AO, TILE>(P, sms, s);
     }
-    if (P.n_part > 4 * P.n_groups) {
-        // (fewer particles: even a group that meets all of them is done before
-        // the others; lens fit, 1e5 particles, 31,250 groups)
-        const uint32_t* sub = (const uint32_t*)(base + L.sub);
-        WalkParams<T> Q = P;
-        Q.sub = sub + 16;
-        Q.sub_n = sub;
-        walk_rounds<T, R>(Q, P.n_groups, nq, base, L, counter, cut, cut_warps, s);
-        P.gflag = (const uint8_t*)(base + L.gflag);
-        P.skip = 1;
-        cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
-        P.counter = counter;
-    }
-    launch_plain<KIND, T, R, AO, TILE>(P, sms, s);
 }
 
 template <typename T, int R>
@@ -1247,6 +1290,7 @@ static lens_status enqueue_typed(lens_tree* t, const ShootPlan& plan, const void
     P.stats = (flags & LENS_COUNT) ? t->d_stats : nullptr;
     P.gH = gH; P.gbox = gbox; P.grange = grange; P.ray_l = ray_l; P.ray_idx = ray_idx;
     P.n_groups = (int64_t)ng;
+    P.n_rays = n;
     P.stack = stack;
     P.err = t->d_err;
     P.wait_cycles = t->wait_cycles;

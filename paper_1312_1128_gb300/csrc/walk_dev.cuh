@@ -118,6 +118,7 @@ template <typename T> struct WalkParams : EvalConsts<T> {
     const v2_t<T>* gH;
     const vec4_t<T>* gbox;
     const uint2* grange;
+    int64_t n_rays;
     const v2_t<T>* ray_l;
     const uint32_t* ray_idx;
     int64_t n_groups;
@@ -147,7 +148,7 @@ template <typename T> struct WalkParams : EvalConsts<T> {
     int list_K;
     CutParams<T> cut;  // parts of groups whose walk is shared by several warps
     const uint8_t* gflag;     // per group: 1 if stretched (walk_shared.cuh)
-    // only the groups sub[0 .. *sub_n) (null: all), or all but the stretched ones
+    // only the groups sub[0 .. *sub_n) (null: all); skip: all but the stretched ones
     const uint32_t* sub;
     const uint32_t* sub_n;
     int skip;
@@ -279,6 +280,7 @@ template <int KIND, typename T, int TILE = 0, int NR = 2> struct PlainShared {
     WalkBuf<KIND, T, TILE> buf;
     WalkRanges rng;
     WalkTot<T, NR> tot;
+    WalkCut cut;
 };
 
 // Room in the totals for R rays per lane.
@@ -779,7 +781,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0, bool LOC = false> 
     using Buf = WalkBuf<KIND, T, TILE>;
     using Flush = WalkFlush<KIND, T, R, AO, TILE, LOC>;
     static constexpr int kKind = KIND, kR = R;
-    static constexpr bool kCuts = true;
+    static constexpr bool kCuts = true, kDefer = true;  // may be cut; puts long lists aside
     static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
     const WalkParams<T>& P;
     typename Flush::WS& S;
@@ -838,7 +840,7 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0, bool LOC = false> 
         if constexpr (LOC) {
             local_zero(S.loc.sum);
             if (lane == 0) {
-                S.loc.rho2 = P.super && P.super[Cut->g / kSuperGroups].ok == 2 ? -1.0f : kLocRho2;
+                S.loc.rho2 = P.super && P.super[Cut->g / kSuperGroups].ok >= 2 ? -1.0f : kLocRho2;
                 S.loc.d = local_scale(box.z, box.w, P.node_rcm[0]);
             }
         }
@@ -868,17 +870,18 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0, bool LOC = false> 
     }
 };
 
-// The context of the plain walk kernel (no cuts, no expansions): the rays stay
-// in registers and full buffers are evaluated inline.
-template <int KIND, typename T, int R, bool AO, int TILE = 0> struct PlainCtx : WalkEval<KIND, T, R, AO, TILE> {
+// The context of the plain walk kernel (whole groups, no expansions): the rays
+// stay in registers and full buffers are evaluated inline.  With CUTS a heavy
+// group's walk may end in a cut, but no list is put aside for it.
+template <int KIND, typename T, int R, bool AO, int TILE, bool CUTS> struct PlainCtx : WalkEval<KIND, T, R, AO, TILE> {
     using value_type = T;
     using Buf = WalkBuf<KIND, T, TILE>;
     static constexpr int kKind = KIND, kR = R;
-    static constexpr bool kCuts = false;
+    static constexpr bool kCuts = CUTS, kDefer = false;
     static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
     const WalkParams<T>& P;
     WalkRanges* Rg;
-    WalkCut* Cut = nullptr;
+    WalkCut* Cut;
     // boxes visited, cells accepted, leaf particles, big entries scanned, kept
     uint32_t c_vis = 0, c_acc = 0, c_near = 0, c_bigs = 0, c_bigk = 0;
     int nf = 0, nn = 0, nb = 0;
@@ -886,8 +889,8 @@ template <int KIND, typename T, int R, bool AO, int TILE = 0> struct PlainCtx : 
     uint32_t* rec_shared = nullptr;
     int rec_n = 0, rec_cap = 0;
 
-    LENS_DEV PlainCtx(const WalkParams<T>& p, Buf* b, WalkTot<T, tot_rays<R>()>* t, WalkRanges* r)
-        : WalkEval<KIND, T, R, AO, TILE>(p, b, t), P(p), Rg(r) {}
+    LENS_DEV PlainCtx(const WalkParams<T>& p, Buf* b, WalkTot<T, tot_rays<R>()>* t, WalkRanges* r, WalkCut* c)
+        : WalkEval<KIND, T, R, AO, TILE>(p, b, t), P(p), Rg(r), Cut(c) {}
     LENS_DEV void flush_far()
     {
         this->eval_far(nf);
@@ -1079,25 +1082,27 @@ template <int R, typename T> LENS_DEV unsigned char* cut_own(const CutParams<T>&
 // Cut the walk: the boxes at the bottom of the stack (the shallowest) and the
 // deferred lists go to a slot of the pool, or stay in the warp's own if the
 // pool is full.  Returns how many boxes stay (at the bottom of the stack).
-template <int R, typename T> LENS_DEV int cut_now(const CutParams<T>& cp, WalkCut& K, int* stack, int sp)
+// DEFER: the walk puts lists aside (one that does not has no slot of its own,
+// and is only cut where every group has a place: cuts_fit).
+template <int R, bool DEFER = true, typename T> LENS_DEV int cut_now(const CutParams<T>& cp, WalkCut& K, int* stack, int sp)
 {
     const uint32_t lane = threadIdx.x & 31;
     const CutPool<T>& pool = cp.out;
-    const bool part = K.local;  // a part that the warp walks itself
+    const bool part = DEFER && K.local;  // a part that the warp walks itself
     uint32_t ci = 0;
     if (lane == 0 && !part) ci = atomicAdd(pool.cnt, 1u);
     ci = __shfl_sync(0xffffffffu, ci, 0);
-    const bool pooled = !part && ci < pool.max_cuts;
-    CutSlot* own = K.own;
+    const bool pooled = !DEFER || (!part && ci < pool.max_cuts);
+    CutSlot* own = DEFER ? K.own : nullptr;
     CutSlot* s = pooled ? pool.slots + ci : own;
     const int nd = sp < kCutNodes ? sp : kCutNodes;
-    if (pooled)
+    if (DEFER && pooled)
         for (int i = (int)lane; i < K.n_ranges; i += 32) s->ranges[i] = own->ranges[i];
     for (int i = (int)lane; i < nd; i += 32) s->nodes[i] = stack[i];
     if (lane == 0) {
         s->g = K.g;
         s->n_nodes = (uint32_t)nd;
-        s->n_ranges = (uint32_t)K.n_ranges;
+        s->n_ranges = DEFER ? (uint32_t)K.n_ranges : 0u;
         s->parent = K.item == kNoItem ? -1 : (int32_t)K.item;
         if (part) {
             K.sub = 1;
@@ -1128,6 +1133,8 @@ template <int R, typename T> LENS_DEV int cut_now(const CutParams<T>& cp, WalkCu
 // lists are put aside, and once the walk has evaluated `limit` entries (or
 // has only long lists left) it is cut.  The deferred lists of the item itself
 // (C.Cut->rn) are scanned 32 to a step, in steps without boxes.
+// A context that puts no lists aside stops there instead, the boxes left on the
+// stack (C.Cut->sp).
 // Returns false if the warp's stack overflowed (the error word is set).
 template <class Ctx, typename T = typename Ctx::value_type>
 LENS_DEV bool traverse(Ctx& C, int* stack, int sp)
@@ -1136,11 +1143,11 @@ LENS_DEV bool traverse(Ctx& C, int* stack, int sp)
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const WalkParams<T>& P = C.P;
-    uint32_t limit = Ctx::kCuts ? C.Cut->limit : kNoCut;
-    int rn = Ctx::kCuts ? C.Cut->rn : 0;
+    uint32_t limit = Ctx::kDefer ? C.Cut->limit : kNoCut;
+    int rn = Ctx::kDefer ? C.Cut->rn : 0;
     for (;;) {
         bool lists = false;  // a step of deferred lists
-        if constexpr (Ctx::kCuts && KIND != LENS_POINT) {
+        if constexpr (Ctx::kDefer && KIND != LENS_POINT) {
             lists = rn > 0;
             if (sp == 0 && !lists && limit != kNoCut && C.Cut->n_ranges > 0) {
                 // only deferred lists are left: worth a cut (a list's chunk
@@ -1222,7 +1229,7 @@ LENS_DEV bool traverse(Ctx& C, int* stack, int sp)
                 if (!big) Lk.w = 0;
             }
             if (Lk.w > 0 && (lists || big)) cnt = ((Lk.z + Lk.w - 1) >> 5) - (Lk.z >> 5) + 1;
-            if constexpr (Ctx::kCuts) {
+            if constexpr (Ctx::kDefer) {
                 if (!lists && limit != kNoCut) {
                     const bool put = cnt > (P.cut.defer ? 0 : kLongList);
                     const unsigned bm = __ballot_sync(full, put);
@@ -1253,9 +1260,17 @@ LENS_DEV bool traverse(Ctx& C, int* stack, int sp)
         }
         if constexpr (Ctx::kCuts) {
             const uint32_t work = C.c_near + C.c_bigk + (C.c_acc >> 1) + (C.c_bigs >> 4);
-            if (work >= limit && sp >= C.Cut->min_nodes) {
-                sp = cut_now<Ctx::kR>(P.cut, *C.Cut, stack, sp);
-                limit = kNoCut;
+            if constexpr (Ctx::kDefer) {
+                if (work >= limit && sp >= C.Cut->min_nodes) {
+                    sp = cut_now<Ctx::kR>(P.cut, *C.Cut, stack, sp);
+                    limit = kNoCut;
+                }
+            } else if (work >= C.Cut->limit && sp >= C.Cut->min_nodes && sp <= kCutNodes) {
+                // (the kernel cuts once the buffers are flushed: the code of
+                // the cut in here cost it registers)
+                if (lane == 0) C.Cut->sp = sp;
+                __syncwarp();
+                break;
             }
         }
     }
@@ -1277,6 +1292,29 @@ LENS_DEV void load_part(WalkCut& K, int* stack)
     __syncwarp();
 }
 
+// The work after which group g is cut (kNoCut: never).
+template <typename T> LENS_DEV uint32_t cut_limit(const WalkParams<T>& P, uint32_t g)
+{
+    const CutParams<T>& cp = P.cut;
+    if (!cp.out.cnt) return kNoCut;
+    return cp.limit_stretched && P.gflag[g] ? cp.limit_stretched : cp.limit;
+}
+
+// A whole group for a kernel without parts: the root on the stack.
+template <typename T> LENS_DEV void whole_group(const WalkParams<T>& P, WalkCut& K, uint32_t g, int* stack)
+{
+    if ((threadIdx.x & 31) == 0) {
+        K.g = g;
+        K.item = kNoItem;
+        K.limit = cut_limit(P, g);
+        K.min_nodes = P.cut.min_nodes;
+        K.fired = K.local = 0;
+        K.sp = 0;
+        stack[0] = 0;
+    }
+    __syncwarp();
+}
+
 // Take the next item (false: none left); its boxes go on the stack.
 template <int R, typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int* stack, WalkCut& K)
 {
@@ -1287,53 +1325,50 @@ template <int R, typename T> LENS_DEV bool next_item(const WalkParams<T>& P, int
     const int64_t n = in.cnt ? (int64_t)cuts * parts
                       : P.sub ? (int64_t)*P.sub_n
                       : P.super && P.super[0].ok == 3 ? 0 : P.n_groups;
-    for (;;) {
-        uint32_t item = 0;
-        if (lane == 0) item = atomicAdd(P.counter, 1u);
-        item = __shfl_sync(full, item, 0);
-        if ((int64_t)item >= n) return false;
-        if (!in.cnt && P.skip && P.gflag[P.order ? P.order[item] : item]) continue;
-        if (lane == 0) {
-            K.limit = !P.cut.out.cnt ? kNoCut : P.cut.limit << (parts < P.cut.few_parts ? 2 : 0);
-            K.min_nodes = P.cut.min_nodes;
-            K.n_ranges = 0;
-            K.chunks = 0;
-            K.fired = K.local = 0;
-            K.seg = K.sub = 0;
-            K.own = (CutSlot*)cut_own<R>(P.cut);
-            K.rn = 0;
-            if (in.cnt) {
-                const CutSlot* cs = in.slots + item / parts;
-                K.cs = cs;
-                K.j = (int)(item % parts);
-                K.parts = (int)parts;
-                K.g = cs->g;
-                K.item = item;
-            } else {
-                K.cs = nullptr;
-                K.g = P.sub ? P.sub[item] : P.order ? P.order[item] : item;
-                if (P.cut.limit_stretched && P.cut.out.cnt && P.gflag[K.g]) K.limit = P.cut.limit_stretched;
-                K.item = kNoItem;
-                K.sp = 1;
-                stack[0] = 0;
-            }
-        }
-        __syncwarp();
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(P.counter, 1u);
+    item = __shfl_sync(full, item, 0);
+    if ((int64_t)item >= n) return false;
+    if (lane == 0) {
+        K.min_nodes = P.cut.min_nodes;
+        K.n_ranges = 0;
+        K.chunks = 0;
+        K.fired = K.local = 0;
+        K.seg = K.sub = 0;
+        K.own = (CutSlot*)cut_own<R>(P.cut);
+        K.rn = 0;
         if (in.cnt) {
-            load_part(K, stack);
-        } else if (P.super) {
-            // the boxes that the supergroup's walk left
-            const SuperRec& sr = P.super[K.g / kSuperGroups];
-            if (sr.ok == 1) {
-                const int n = sr.n;
-                for (int i = lane; i < n; i += 32) stack[i] = sr.nodes[i];
-                __syncwarp();
-                if (lane == 0) K.sp = n;
-                __syncwarp();
-            }
+            const CutSlot* cs = in.slots + item / parts;
+            K.cs = cs;
+            K.j = (int)(item % parts);
+            K.parts = (int)parts;
+            K.g = cs->g;
+            K.limit = !P.cut.out.cnt ? kNoCut : P.cut.limit << (parts < P.cut.few_parts ? 2 : 0);
+            K.item = item;
+        } else {
+            K.cs = nullptr;
+            K.g = P.sub ? P.sub[item] : P.order ? P.order[item] : item;
+            K.limit = cut_limit(P, K.g);
+            K.item = kNoItem;
+            K.sp = 1;
+            stack[0] = 0;
         }
-        return true;
     }
+    __syncwarp();
+    if (in.cnt) {
+        load_part(K, stack);
+    } else if (P.super) {
+        // the boxes that the supergroup's walk left
+        const SuperRec& sr = P.super[K.g / kSuperGroups];
+        if (sr.ok == 1) {
+            const int n = sr.n;
+            for (int i = lane; i < n; i += 32) stack[i] = sr.nodes[i];
+            __syncwarp();
+            if (lane == 0) K.sp = n;
+            __syncwarp();
+        }
+    }
+    return true;
 }
 
 // A cut whose pool was full: after each segment (the item's own, then each
@@ -1463,47 +1498,90 @@ __global__ void k_cut_sum(CutPool<T> pool, CutPool<T> to, WalkParams<T> P, int n
     }
 }
 
-// The launches of one tree walk over ng groups: `walk(P)` launches the
-// kernel, of `warps` warps.  Groups are cut in a launch's kernel and their parts
-// run in the next one; a part may be cut once more.  Launches without items
-// cost about 3 us each, beside walks of 100 us and more.
-//   ng <= 512: far fewer warps than the chip holds.  Every group is cut as
-//     soon as its stack holds 64 boxes (its big lists deferred to the parts),
-//     into enough parts for about 8,192 warps.
-//   ng <= 4096: a group is cut after a share of work that about doubles the
-//     launch's warps.
-//   above: only a group far heavier than the others (16,384 entries and more;
-//     an average one evaluates 5,000 to 7,000), or a stretched one (which may
-//     hold most of the tree) beyond 8,192; the fewer they are, the more parts.
-//     Where the groups are more than the pool has room for, 8 parts each.
-//   keep_order (FP32 point masses): none but the heavy ones.  Over a patch much
-//     smaller than the distances all rays share the rounding of one sum of
-//     thousands of terms, which shows in a component that happens to be small
-//     (1e-3 of the sum of |terms|): such groups keep their order of summation.
-template <typename T, int R, typename Walk>
-void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& L, uint32_t* counter, Walk&& walk,
-                 int warps, cudaStream_t s, bool keep_order = false)
+// How the groups of a tree walk are cut (walk_rounds).
+struct CutPlan {
+    bool few;         // all groups are cut, their long lists put aside from the start
+    bool keep_order;  // FP32 point masses: only the heaviest
+    bool stretched;   // the call's stretched groups alone (P.sub): all of them
+};
+constexpr int64_t kFewGroups = 4096;
+
+// Is no group of a tree of n particles worth a cut (five more launches)?  Times
+// with cuts, and without:
+//   few groups: 400 particles, 100 to 1e5 rays 1.05 to 1.15 times as long; 700
+//     particles, 100 rays 0.22 ms, 0.29; FP64, 400 particles, 1,000 rays 0.59 ms,
+//     0.69.  Above 512 groups the groups are many beside the particles at first
+//     (3,750 groups, 1,200 particles 0.40 ms, 0.39; 5,000 particles 0.63, 0.81).
+//     One ray: 700 particles 0.126 ms, 0.100; 2,500 particles 0.113, 0.128.
+//   others: no walk is longer than 2 n + n / 16 entries (cells and leaf particles,
+//     listed ones, their tests); 0.3 ms for 16,384 entries.  Point masses, theta
+//     0.3: 1e5 particles 0.69 ms, 0.63; 3e5: 0.95, 1.08; theta 0.1 (9 times the
+//     entries): 84,000 particles in 144 batches 6.5, 10.0.
+inline bool never_cut(const lens_tree* t, int64_t ng, int64_t n_rays, int64_t n, const CutPlan& plan)
+{
+    const bool fp64 = t->precision == LENS_PREC_FP64;
+    if (plan.few) return n <= (fp64 ? 256 : 512) || (ng > 512 && n <= ng) || (n_rays == 1 && n < 1024);
+    const double th = std::min(t->theta / 0.3, 1.0);
+    return plan.keep_order ? n < 8192 || n < 131072 * th * th : 2 * n + n / 16 < 16384;
+}
+
+// Room for the first pool of a walk's cuts, and whether every one of ng groups
+// has a place there.
+template <typename T, int R> size_t cut_room(const Layout& L, int warps, int cut_warps)
+{
+    constexpr size_t total = 5 * 32 * R * sizeof(T), again = kCutAgainBytes / 16 * (16 + 1) + kCutAgainBytes / (16 * total) * sizeof(CutSlot);
+    return L.cut_end - L.stack - (size_t)warps * kStackCap * sizeof(int) -
+           (size_t)cut_warps * 2 * cut_local_bytes<R, T>() - again - 8 * 256;
+}
+template <typename T, int R> bool cuts_fit(int64_t ng, const Layout& L, int warps, int cut_warps)
+{
+    return (size_t)ng * (sizeof(CutSlot) + 2 * 5 * 32 * R * sizeof(T)) <= cut_room<T, R>(L, warps, cut_warps);
+}
+
+// The launches of one tree walk over ng groups: `groups(P)` launches the kernel
+// for whole groups, `parts(P)` the one for parts.  Groups are cut in a launch's
+// kernel and their parts run in the next one; a part may be cut once more.
+// Launches without items cost about 3 us each, beside walks of 100 us and more.
+// warps: of the kernel with the most; cut_warps: of the cut form.
+//   few (up to 4,096 groups): about as many warps as the chip holds, or fewer.
+//     Up to 512 groups are cut as soon as their stack holds 64 boxes (their big
+//     lists deferred to the parts), into enough parts for about 8,192 warps; up
+//     to 4,096 after a share of work that about doubles the launch's warps.
+//   stretched: some tens or hundreds, cut as up to 512 groups are.
+//   otherwise: only a group far heavier than the others (16,384 entries and
+//     more; an average one evaluates 5,000 to 7,000), or a stretched one (which
+//     may hold most of the tree) beyond 8,192; the fewer they are, the more
+//     parts.  Where the groups are more than the pool has room for, 8 parts each.
+//   keep_order (FP32 point masses): never few.  Over a patch much smaller than
+//     the distances all rays share the rounding of one sum of thousands of
+//     terms, which shows in a component that happens to be small (1e-3 of the
+//     sum of |terms|): such groups keep their order of summation.
+template <typename T, int R, typename Groups, typename Parts>
+void walk_rounds(WalkParams<T> P, const CutPlan& plan, int nq, char* base, const Layout& L, uint32_t* counter,
+                 Groups&& groups, Parts&& parts, int warps, int cut_warps, cudaStream_t s)
 {
     // counter: 8 words, zeroed by the caller: work counters, then each pool's
     CutPool<T> pool[2];
     constexpr size_t total = 5 * 32 * R * sizeof(T);
+    const int64_t ng = P.n_groups;
+    const bool few = plan.few;
     char* at = base + L.stack + (size_t)warps * kStackCap * sizeof(int);
     auto take = [&](size_t bytes) {
         char* p = at;
         at += (bytes + 255) & ~(size_t)255;
         return p;
     };
+    // (twice: where the first pool may be full)
     const size_t local_bytes = cut_local_bytes<R, T>() * 2;
-    unsigned char* local = (unsigned char*)take((size_t)warps * local_bytes);
+    unsigned char* local = (unsigned char*)take((size_t)cut_warps * local_bytes);
     // the second pool: parts that are cut again
-    pool[1].parts = ng <= 4096 && !keep_order ? 16 : 32;
+    pool[1].parts = few || plan.stretched ? 16 : 32;
     pool[1].max_cuts = (uint32_t)(kCutAgainBytes / (pool[1].parts * total));
     pool[1].slots = (CutSlot*)take(pool[1].max_cuts * sizeof(CutSlot));
     pool[1].head = (T*)take(pool[1].max_cuts * total);
     pool[1].part = (T*)take(pool[1].max_cuts * pool[1].parts * total);
     // the first has the rest: every group that may be cut has a place
-    const size_t room = (size_t)(base + L.cut_end - at) - 4 * 256;
-    const bool few = ng <= 4096 && !keep_order;
+    const size_t room = cut_room<T, R>(L, warps, cut_warps);
     bool all = true;
     if (few) {
         const size_t fit = (room - (size_t)ng * (sizeof(CutSlot) + total)) / total;
@@ -1512,9 +1590,9 @@ void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& 
         pool[0].items = (uint32_t)std::min<size_t>(ng <= 512 ? 8192 : 28672, fit);
     } else {
         // a place for every group, or 8 parts each for as many as fit
-        all = (size_t)ng * (sizeof(CutSlot) + 2 * total) <= room;
+        all = cuts_fit<T, R>(ng, L, warps, cut_warps);
         pool[0].max_cuts = (uint32_t)(all ? (size_t)ng : room / (sizeof(CutSlot) + 9 * total));
-        pool[0].parts = all ? 32 : 8;
+        pool[0].parts = all ? plan.stretched ? 64 : 32 : 8;
         pool[0].items = all ? (uint32_t)std::min<size_t>(28672, (room - pool[0].max_cuts * (sizeof(CutSlot) + total)) / total) : 0;
     }
     pool[0].slots = (CutSlot*)take(pool[0].max_cuts * sizeof(CutSlot));
@@ -1535,8 +1613,15 @@ void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& 
         c[0].min_nodes = 32;
         c[1].limit = c[0].limit;
         c[1].min_nodes = 16;
+    } else if (plan.stretched) {
+        c[0].limit = 0;
+        c[0].min_nodes = 64;
+        c[0].defer = 1;
+        c[1].limit = 512;
+        c[1].few_parts = 32;  // (over 896 groups)
+        c[1].min_nodes = 16;
     } else {
-        c[0].limit = (uint32_t)(ng <= 10922 || keep_order ? 16384 : 3 * (ng / 2));
+        c[0].limit = (uint32_t)(ng <= 10922 || plan.keep_order ? 16384 : 3 * (ng / 2));
         c[0].limit_stretched = 8192;
         c[0].min_nodes = 32;
         c[1].limit = 8192;
@@ -1553,7 +1638,8 @@ void walk_rounds(WalkParams<T> P, int64_t ng, int nq, char* base, const Layout& 
         if (r > 0) c[r].in = pool[r - 1];
         if (r + 1 < rounds) c[r].out = pool[r];
         P.cut = c[r];
-        walk(P);
+        if (r == 0) groups(P);
+        else parts(P);
     }
     for (int r = rounds - 2; r >= 0; --r) {
         const int64_t most = std::min<int64_t>(pool[r].max_cuts, r > 0 ? 2048 : ng);

@@ -63,10 +63,7 @@ constexpr size_t kCutSlotBytes = 2320;
 // fill power-of-two squares a few groups span half the map and open most of
 // the tree (one warp then walked on for 18 of 20 ms at 700^2 rays through 3e5
 // particles).  A group is stretched if a side of its box is over kStretch
-// times that of an even share of its batch.  From kPlainGroups groups on a
-// walk takes them in launches of their own, where they are cut early
-// (walk_dev.cuh), and the others in the plain kernel.
-constexpr int64_t kPlainGroups = 24576;
+// times that of an even share of its batch.
 constexpr float kStretch = 16.0f;
 
 // Supergroups (walk_dev.cuh): kSuperGroups consecutive groups, one record each.

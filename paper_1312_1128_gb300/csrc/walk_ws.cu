@@ -99,7 +99,7 @@ template <int KIND, typename T, int CONS> struct WsProducer {
     using value_type = T;
     using Buf = WalkBuf<KIND, T>;
     static constexpr int kKind = KIND, kR = 1;
-    static constexpr bool kCuts = false;  // (the team's slots go to its consumers)
+    static constexpr bool kCuts = false, kDefer = false;  // (the team's slots go to its consumers)
     static constexpr int kNear = Buf::kNear, kBig = Buf::kBig;
     const WalkParams<T>& P;
     WsPair<KIND, T, CONS>& W;

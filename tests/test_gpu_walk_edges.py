@@ -112,3 +112,127 @@ def test_scratch_of_a_small_lens():
     for lens in lenses:
         lens.close()
     assert used <= 8 * 200e6, used / 8
+
+
+def ray_groups(dx, dy, group):
+    """The rays of each group (Morton order of 16-bit positions in their box)
+    and the groups whose box is stretched: a side over 16 times that of an
+    even share of the rays' box."""
+    x0, y0 = dx.min(), dy.min()
+    wx, wy = dx.max() - x0, dy.max() - y0
+    inv = 65535.99 / max(wx, wy)
+
+    def spread(v):
+        v = v.astype(np.uint64)
+        for s, m in ((8, 0x00ff00ff), (4, 0x0f0f0f0f), (2, 0x33333333), (1, 0x55555555)):
+            v = (v | (v << np.uint64(s))) & np.uint64(m)
+        return v
+
+    keys = spread(np.floor((dx - x0) * inv)) | (spread(np.floor((dy - y0) * inv)) << np.uint64(1))
+    order = np.argsort(keys, kind="stable")
+    groups = [order[i:i + group] for i in range(0, order.size, group)]
+    share = np.sqrt(group / dx.size)
+    stretched = [g for g in groups if np.ptp(dx[g]) > 16 * share * wx or np.ptp(dy[g]) > 16 * share * wy]
+    return groups, stretched
+
+
+def outside_a_disk(n):
+    """A grid of rays without a disk in its middle: Morton-consecutive rays
+    across the hole make groups that span it."""
+    rx, ry = lensgen.grid_rays(n, -1.0, 1.0, dtype=np.float32)
+    m = rx ** 2 + ry ** 2 > 0.3
+    return rx[m], ry[m]
+
+
+@pytest.mark.parametrize("form", ["gauss", "gauss_alpha", "gauss_64", "gauss_fp64", "few_particles", "cut_form", "potential"])
+def test_stretched_groups_are_cut(form):
+    """Stretched groups in the launches that cut them: from 24,576 groups on (or
+    with fewer than 24,576 particles) by themselves while the plain kernel takes
+    the others, below with all groups; more than four particles a group.
+    Reference: the producer/consumer form, 1e-6 of the sum of |terms| (1e-14 in
+    FP64; the potential's: its direct evaluation of those rays alone, which cuts
+    its one group per call into parts)."""
+    from lens_testutil import comps_gauss
+    group = 64 if form == "gauss_64" else 32
+    n = 23_000 if form == "few_particles" else 172_000
+    dx, dy = outside_a_disk(1800 if form == "gauss_64" else 480 if form == "few_particles" else
+                            900 if form in ("cut_form", "potential") else 1300)
+    groups, stretched = ray_groups(dx, dy, group)
+    if form not in ("cut_form", "potential"):
+        assert len(groups) >= 24576 or (4096 < len(groups) and n < 24576)
+    else:
+        assert 4096 < len(groups) < 24576
+    assert n > 4 * len(groups) and len(stretched) > 0
+    p = lensgen.nfw_particles(n, 9, nsph=32)
+    prec = "fp64" if form == "gauss_fp64" else "fp32"
+    dt = np.float64 if prec == "fp64" else np.float32
+    dx, dy = dx.astype(dt), dy.astype(dt)
+    lens = L.Lens([L.Species.gauss(cu(p), 3.0)], theta=0.3, group_rays=group, precision=prec)
+    ref = L.Lens([L.Species.gauss(cu(p), 3.0)], theta=0.3, group_rays=group, precision=prec, walk="pairs")
+    widest = max(stretched, key=lambda g: np.ptp(dx[g]) + np.ptp(dy[g]))
+    lens.shoot(cu(dx[widest]), cu(dy[widest]), flags=L.COUNT)
+    c = lens.counters()
+    assert c["cells"] // 2 + c["leaf_particles"] + c["big_kept"] > 8192  # (the least a cut takes)
+    idx = np.unique(np.concatenate(stretched[:8] + [widest] + [groups[0], groups[-1]]))
+    flags = L.ALPHA_ONLY if form == "gauss_alpha" else 0
+    if form == "potential":
+        got = np.stack([o.double().cpu().numpy()[idx] for o in lens.potential(cu(dx), cu(dy))], 1)
+        want = np.stack([o.double().cpu().numpy() for o in ref.potential(cu(dx[idx]), cu(dy[idx]))], 1)
+        # (other groups take other decisions near a cell's radius: the tree's
+        # own accuracy at theta 0.3)
+        assert (np.abs(got - want).max(0) / np.abs(want).max(0)).max() <= 1e-3
+    else:
+        got, want = (np.stack([o.double().cpu().numpy()[idx] for o in q.shoot(cu(dx), cu(dy), flags=flags) if o is not None], 1)
+                     for q in (lens, ref))
+        _, absum = oracle.direct_sum(comps_gauss(p, 3.0), dx[idx].astype(np.float64), dy[idx].astype(np.float64), with_absum=True)
+        d = np.abs(got - want) / (absum[:, :got.shape[1]] + 1e-300)
+        assert d.max() <= (1e-14 if prec == "fp64" else 1e-6)
+    lens.close()
+    ref.close()
+
+
+def test_adjoint_after_cut_groups():
+    """The lists kept by parts of stretched groups give the walk's gradients."""
+    g = lensgen.rng(3)
+    dx, dy = outside_a_disk(1300)
+    p = lensgen.nfw_particles(172_000, 9, nsph=32)
+    a, b = (cu((0.01 * g.standard_normal(dx.size)).astype(np.float32)) for _ in range(2))
+    lens = L.Lens([L.Species.gauss(cu(p), 3.0)], theta=0.3, group_rays=32)
+    x, y = cu(dx), cu(dy)
+    (walked,) = lens.backward(x, y, a, b)
+    lens.shoot(x, y, flags=L.ALPHA_ONLY | L.KEEP_LISTS)
+    (replayed,) = lens.backward(x, y, a, b, flags=L.KEEP_LISTS)
+    for k in range(4):
+        assert (replayed[:, k] - walked[:, k]).abs().max() <= 1e-6 * walked[:, k].abs().max()
+    lens.close()
+
+
+@pytest.mark.parametrize("kind", ["gauss", "nfw", "points", "points_fp64"])
+@pytest.mark.parametrize("groups", [1, 2, 512, 513, 4096, 4097])
+def test_group_counts_at_the_rules(kind, groups):
+    """Group counts next to the rules, full groups and one ray more than the
+    count before; trees of 1,000 and 20,000 particles (fewer than 512 are not
+    cut).  1e-6 of the sum of |terms| (FP64: 1e-14)."""
+    from lens_testutil import comps_gauss
+    g = lensgen.rng(groups)
+    prec = "fp64" if kind == "points_fp64" else "fp32"
+    dt = np.float64 if prec == "fp64" else np.float32
+    for n, rays in ((1000, 32 * groups), (20000 if kind != "nfw" else 3000, 32 * (groups - 1) + 1)):
+        if kind == "gauss":
+            p = lensgen.nfw_particles(n, 7, nsph=32)
+            species, comps = L.Species.gauss(cu(p), 3.0), comps_gauss(p, 3.0)
+        elif kind == "nfw":
+            p = lensgen.nfw_test_halos(n, 22, 0.3)
+            species, comps = L.Species.nfw(cu(p), 3.0), comps_nfw(p, 3.0)
+        else:
+            p = lensgen.point_disk(n, 33)
+            species, comps = L.Species.points(cu(p)), comps_points(p)
+        dx, dy = (g.uniform(-0.9, 0.9, rays).astype(dt) for _ in range(2))
+        out = []
+        for walk in ("warp", "pairs"):
+            lens = L.Lens([species], theta=0.3, precision=prec, group_rays=32, walk=walk)
+            out.append(np.stack([o.double().cpu().numpy() for o in lens.shoot(cu(dx), cu(dy))], 1))
+            lens.close()
+        idx = np.unique(np.r_[0, rays - 1, g.integers(0, rays, 60)])
+        _, absum = oracle.direct_sum(comps, dx[idx].astype(np.float64), dy[idx].astype(np.float64), with_absum=True)
+        assert (np.abs(out[0][idx] - out[1][idx]) / (absum + 1e-300)).max() <= (1e-14 if prec == "fp64" else 1e-6)
