@@ -567,13 +567,13 @@ static lens_status psi_typed(lens_tree* t, const ShootPlan& plan, const void* dx
                 constexpr int R = decltype(rays)::value;
                 auto cut = [&](const WalkParams<T>& Q) { psi_launch_kind<T, R, 2>(kind, Q, K, t->num_sms, s); };
                 auto whole = [&](const WalkParams<T>& Q) { psi_launch_kind<T, R, 1>(kind, Q, K, t->num_sms, s); };
-                // few groups, and mid-sized calls of larger trees: the cut
-                // form; otherwise whole groups, whose kernel has 16 to 24
-                // registers less (20,000 particles: 1.04 to 1.2 times as fast)
+                // the cut form; small trees' whole groups by a kernel with 16 to
+                // 24 registers less (20,000 particles 1.04 to 1.2 times as fast;
+                // 300,000 particles, 25,992 groups 9.0 ms, the cut form 7.7)
                 const CutPlan cp{ng <= kFewGroups, false, false};
                 const int cut_warps = psi_warps<T, R, 2>(kind, t->num_sms);
                 const int warps = std::max(cut_warps, psi_warps<T, R, 1>(kind, t->num_sms));
-                const bool cuts = cp.few || (ng < 24576 && P.n_part >= 24576) || !cuts_fit<T, R>(ng, L, warps, cut_warps);
+                const bool cuts = cp.few || P.n_part >= 24576 || !cuts_fit<T, R>(ng, L, warps, cut_warps);
                 if (never_cut(t, ng, P.n_rays, P.n_part, cp)) whole(P);
                 else if (cuts) walk_rounds<T, R>(P, cp, 3, base, L, P.counter, cut, cut, cut_warps, cut_warps, s);
                 else walk_rounds<T, R>(P, cp, 3, base, L, P.counter, whole, cut, warps, cut_warps, s);

@@ -489,6 +489,10 @@ walk_plain(const __grid_constant__ WalkParams<T> P)
     int* stack = P.stack + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
     PlainCtx<KIND, T, R, AO, TILE, CUTS> C(P, &S.buf, &S.tot, &S.rng, &S.cut);
     if (P.super && P.super[0].ok != 3) return;  // the supergroups' walk has run
+    // the rays' indices are read again after the walk where they cost it spills
+    constexpr bool kAgain = CUTS || KIND != LENS_POINT;
+    uint32_t ridx[R];
+    bool rv[R];
     for (;;) {
         uint32_t item = 0;
         if (lane == 0) item = atomicAdd(P.counter, 1u);
@@ -499,16 +503,21 @@ walk_plain(const __grid_constant__ WalkParams<T> P)
         whole_group(P, S.cut, g, stack);
         C.H = P.gH[g];
         C.box = P.gbox[g];
-        const uint2 first = P.grange[g];
+        uint2 rg = P.grange[g];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int k = r * 32 + lane;
-            v2_t<T> l;
-            l.x = C.box.x;
-            l.y = C.box.y;
-            if (k < (int)first.y) l = P.ray_l[first.x + k];
-            C.lx[r] = l.x;
-            C.ly[r] = l.y;
+            rv[r] = k < (int)rg.y;
+            if (rv[r]) {
+                const v2_t<T> l = P.ray_l[rg.x + k];
+                C.lx[r] = l.x;
+                C.ly[r] = l.y;
+                ridx[r] = P.ray_idx[rg.x + k];
+            } else {
+                C.lx[r] = C.box.x;
+                C.ly[r] = C.box.y;
+                ridx[r] = 0;
+            }
             C.part[r].zero();
         }
         C.tot_zero();
@@ -519,23 +528,27 @@ walk_plain(const __grid_constant__ WalkParams<T> P)
         C.rec_cap = P.list_K;
         const bool whole = traverse(C, stack, 1);
         if (C.rec && lane == 0)
-            P.list_n[S.cut.g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListTooLong;
+            P.list_n[kAgain ? S.cut.g : g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListTooLong;
         C.flush_far();
         C.flush_near();
         if constexpr (KIND != LENS_POINT) C.flush_big();
         if (P.n_halos > 0) C.halos(P.halos, P.n_halos);
-        // (read again: kept in registers over the walk they cost it spills)
-        const uint2 rg = P.grange[S.cut.g];
-        count_item(C, S.cut.g, rg.y, true);
+        if constexpr (kAgain) {
+            rg = P.grange[S.cut.g];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                rv[r] = r * 32 + lane < (int)rg.y;
+                ridx[r] = rv[r] ? P.ray_idx[rg.x + r * 32 + lane] : 0u;
+            }
+        }
+        count_item(C, kAgain ? S.cut.g : g, rg.y, true);
         if (CUTS && S.cut.sp > 0) cut_now<R, false>(P.cut, S.cut, stack, S.cut.sp);
         __syncwarp();
         T* tot = CUTS ? item_totals<R>(P.cut, S.cut) : nullptr;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int k = r * 32 + lane;
-            const bool ray = k < (int)rg.y;
-            if (!ray && !tot) continue;
-            const uint32_t i = ray ? P.ray_idx[rg.x + k] : 0u;
+            if (!rv[r] && !tot) continue;
+            const uint32_t i = ridx[r];
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
                 if (AO && q >= 2) break;
@@ -977,9 +990,9 @@ static void launch_direct(int kind, bool ao, const WalkParams<T>& P, int num_sms
 // The one-warp tree walk of all groups.
 //   FP32 NFW trees (expansions) and, up to 4,096 groups, all but FP32 point
 //     masses: the cut form.
-//   FP32 point masses: the plain kernel with cuts (up to 1,024 groups the cut
-//     form: every warp counts there, and its steps are shorter: 504 groups of
-//     67,587 stars 1.11 ms, 1.22).  With supergroups the cut form with
+//   FP32 point masses: the plain kernel with cuts (up to 16 groups per SM the
+//     cut form: more warps than that it can hold too, and its steps are shorter:
+//     504 groups of 67,587 stars 1.11 ms, 1.22; 1,501 of 1.6e6 1.85, 1.98).  With supergroups the cut form with
 //     expansions or, as only the device knows, the plain kernel: the other of
 //     the two launches finds no work.
 //   The others: from kPlainGroups groups on the stretched groups by the cut
@@ -1015,7 +1028,7 @@ static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, co
         const int warps = std::max(cut_warps, kWalkWarps * sms * plain_blocks_per_sm<KIND, T, R, AO, TILE, true>());
         const bool fit = cuts_fit<T, R>(ng, L, warps, cut_warps);
         auto groups = [&](const WalkParams<T>& Q) {
-            const bool whole = fit && ng > 1024;
+            const bool whole = fit && ng > 16 * sms;
             if (Q.super || !whole) cut(Q);
             if (!Q.super && !whole) return;
             WalkParams<T> W = Q;

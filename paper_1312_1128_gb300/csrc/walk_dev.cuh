@@ -1507,29 +1507,38 @@ struct CutPlan {
 constexpr int64_t kFewGroups = 4096;
 
 // Is no group of a tree of n particles worth a cut (five more launches)?  Times
-// with cuts, and without:
+// with cuts, and without, theta 0.3 (at smaller theta a walk meets more of a
+// tree):
 //   few groups: 400 particles, 100 to 1e5 rays 1.05 to 1.15 times as long; 700
 //     particles, 100 rays 0.22 ms, 0.29; FP64, 400 particles, 1,000 rays 0.59 ms,
 //     0.69.  Above 512 groups the groups are many beside the particles at first
 //     (3,750 groups, 1,200 particles 0.40 ms, 0.39; 5,000 particles 0.63, 0.81).
 //     One ray: 700 particles 0.126 ms, 0.100; 2,500 particles 0.113, 0.128.
 //   others: no walk is longer than 2 n + n / 16 entries (cells and leaf particles,
-//     listed ones, their tests); 0.3 ms for 16,384 entries.  Point masses, theta
-//     0.3: 1e5 particles 0.69 ms, 0.63; 3e5: 0.95, 1.08; theta 0.1 (9 times the
-//     entries): 84,000 particles in 144 batches 6.5, 10.0.
+//     listed ones, their tests), of point masses n; 0.3 ms for 16,384 entries.
 inline bool never_cut(const lens_tree* t, int64_t ng, int64_t n_rays, int64_t n, const CutPlan& plan)
 {
-    const bool fp64 = t->precision == LENS_PREC_FP64;
-    if (plan.few) return n <= (fp64 ? 256 : 512) || (ng > 512 && n <= ng) || (n_rays == 1 && n < 1024);
     const double th = std::min(t->theta / 0.3, 1.0);
-    return plan.keep_order ? n < 8192 || n < 131072 * th * th : 2 * n + n / 16 < 16384;
+    const int64_t small = t->precision == LENS_PREC_FP64 ? 256 : 512;
+    if (plan.few)
+        return n <= th * (double)std::max(small, ng > 512 ? ng : 0) || (n_rays == 1 && n < 1024 * th * th);
+    return plan.keep_order ? n < 8192 : 2 * n + n / 16 < 16384;
+}
+
+// Totals in the second pool.  (Twice as many, in 32-ray groups: 400,000
+// particles, 3,750 groups potential 9.4 -> 7.3 ms, 1,046 groups 8.4 -> 12.5: a
+// part whose boxes are one heavy one and 15 light ones gains nothing from a
+// launch of its own, and waits for it.)
+template <typename T, int R> constexpr size_t again_items()
+{
+    return std::min<size_t>(16384, ((size_t)20 << 20) / (5 * 32 * R * sizeof(T)));
 }
 
 // Room for the first pool of a walk's cuts, and whether every one of ng groups
 // has a place there.
 template <typename T, int R> size_t cut_room(const Layout& L, int warps, int cut_warps)
 {
-    constexpr size_t total = 5 * 32 * R * sizeof(T), again = kCutAgainBytes / 16 * (16 + 1) + kCutAgainBytes / (16 * total) * sizeof(CutSlot);
+    constexpr size_t total = 5 * 32 * R * sizeof(T), again = again_items<T, R>() * total + again_items<T, R>() / 17 * sizeof(CutSlot);
     return L.cut_end - L.stack - (size_t)warps * kStackCap * sizeof(int) -
            (size_t)cut_warps * 2 * cut_local_bytes<R, T>() - again - 8 * 256;
 }
@@ -1576,7 +1585,7 @@ void walk_rounds(WalkParams<T> P, const CutPlan& plan, int nq, char* base, const
     unsigned char* local = (unsigned char*)take((size_t)cut_warps * local_bytes);
     // the second pool: parts that are cut again
     pool[1].parts = few || plan.stretched ? 16 : 32;
-    pool[1].max_cuts = (uint32_t)(kCutAgainBytes / (pool[1].parts * total));
+    pool[1].max_cuts = (uint32_t)(again_items<T, R>() / (pool[1].parts + 1));
     pool[1].slots = (CutSlot*)take(pool[1].max_cuts * sizeof(CutSlot));
     pool[1].head = (T*)take(pool[1].max_cuts * total);
     pool[1].part = (T*)take(pool[1].max_cuts * pool[1].parts * total);

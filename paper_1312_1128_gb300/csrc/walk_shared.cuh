@@ -57,7 +57,6 @@ struct Layout {
 // From about 600,000 rays on up to 48 MB are added behind it, so that every
 // group has a place in the first pool up to 24,576 groups.
 constexpr int kWalkBlocks = 8;
-constexpr size_t kCutAgainBytes = (size_t)20 << 20;   // totals of the second pool's parts
 constexpr size_t kCutSlotBytes = 2320;
 // Stretched groups: Morton order jumps between quadrants, so unless the rays
 // fill power-of-two squares a few groups span half the map and open most of
