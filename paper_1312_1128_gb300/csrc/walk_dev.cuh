@@ -1601,7 +1601,7 @@ void walk_rounds(WalkParams<T> P, const CutPlan& plan, int nq, char* base, const
         // a place for every group, or 8 parts each for as many as fit
         all = cuts_fit<T, R>(ng, L, warps, cut_warps);
         pool[0].max_cuts = (uint32_t)(all ? (size_t)ng : room / (sizeof(CutSlot) + 9 * total));
-        pool[0].parts = all ? plan.stretched ? 64 : 32 : 8;
+        pool[0].parts = all ? plan.stretched ? 64 : 16 : 8;
         pool[0].items = all ? (uint32_t)std::min<size_t>(28672, (room - pool[0].max_cuts * (sizeof(CutSlot) + total)) / total) : 0;
     }
     pool[0].slots = (CutSlot*)take(pool[0].max_cuts * sizeof(CutSlot));
