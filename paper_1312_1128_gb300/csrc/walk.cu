@@ -606,13 +606,35 @@ static void launch_plain(const WalkParams<T>& P, int num_sms, cudaStream_t s)
 // group: not worth one warp's time.)
 constexpr uint32_t kSuperWork = 16384;
 constexpr int kSuperLeft = 128, kTinyLeft = 8;      // most boxes left to the groups
-constexpr float kNarrow = 0.01f, kTiny = 1e-6f;     // of the root's r_cm
+// When expansions are taken (one batch; r: the root's r_cm):
+//   Over a patch narrower than kNarrow r the sums of all rays are nearly one
+//     sum, and a component that cancels to 1e-3 of the sum of |terms| is FP32
+//     noise in its fourth digit.  Expanded or not, its error against 64 bits is
+//     the same (rms 3e-8 to 9e-8 of the sum of |terms| from 1e-6 to 0.1 wide),
+//     but the digits are others: up to 2e-4 of alpha2 for 3e6 stars, theta 0.3.
+//     Such patches go to the plain kernel and keep their digits.
+//   Where a group's side is below kTiny r, an eighth of the rounding of a
+//     distance r, all its rays round alike and the correction at the group's
+//     centre (sdelta) gives the plain kernel's digits back (2e-6 to 4e-5 of
+//     alpha2); 4096^2 rays, 1e7 stars over 1e-6: 78 -> 7.7 ms.
+//   Over a wide field nothing is far from a supergroup.  near: the stars in the
+//     zone (of radius d / 0.18) that its expansion cannot stand for, in the mean.
+//     They are evaluated for every ray of 32 R, where the plain kernel evaluates
+//     some number for theta; times of start and supergroups, theta 0.3: R = 1,
+//     near 282: 2.02 -> 1.56 ms, 704: 0.47 -> 0.67; R = 2, 1,131: 1.06 -> 1.03,
+//     2,034: 2.65 -> 2.73; R = 4, 3,973: 4.62 -> 3.89, 7,430: 2.02 -> 2.22.
+//     theta 0.1: R = 1, 990: 2.41 -> 2.14, 7,044: 2.73 -> 2.78, R = 2 and 4
+//     always faster.  Hence 400 R^2 (0.3 / theta)^3 for R = 1 and 2; R = 4 (at
+//     worst 0.91 times as fast, and 1.2 times where groups are stretched): none.
+// Several batches: only the last, for each supergroup by its own d.
+constexpr float kNarrow = 0.01f, kTiny = 7.4505806e-9f;
+constexpr float kNearMax = 400.0f;
 static_assert(kSuperLeft <= kCutNodes, "room in the record");
 constexpr int kLeftBit = 1 << 30;  // (a tree has fewer boxes)
 
 __global__ void __launch_bounds__(kWalkWarps * 32, 4)
 k_super(const __grid_constant__ WalkParams<float> P, const float* rcm, const unsigned long long* bbox,
-        const uint32_t* bb32, SuperRec* rec, float4* sdelta)
+        const uint32_t* bb32, float near_max, SuperRec* rec, float4* sdelta)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using Flush = WalkFlush<LENS_POINT, float, 1, false, 0, true>;
@@ -624,17 +646,19 @@ k_super(const __grid_constant__ WalkParams<float> P, const float* rcm, const uns
     uint8_t* near_left = S.loc.idx + kBigCap;  // near buffer's particles: left to the groups
     int* stack = P.stack + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
     const int64_t n_super = (P.n_groups + kSuperGroups - 1) / kSuperGroups;
-    // One batch over a patch small against the lens: a tiny one, where all
-    // rays of a group share the rounding of their sums, with few boxes left; or
-    // no expansions at all (every ray's sum then keeps its own order, SuperRec).
-    float ext = INFINITY;
-    if (bb32)
-        ext = fmaxf(ordered_to_flt(bb32[2]) - ordered_to_flt(bb32[0]), ordered_to_flt(bb32[3]) - ordered_to_flt(bb32[1]));
-    else if (bbox)
-        ext = (float)fmax(ordered_to_dbl(bbox[1]) - ordered_to_dbl(bbox[0]),
-                             ordered_to_dbl(bbox[3]) - ordered_to_dbl(bbox[2]));
-    const bool narrow = ext < kNarrow * rcm[0];
-    const int most_left = !narrow ? kSuperLeft : ext < kTiny * rcm[0] ? kTinyLeft : -1;
+    float wx = INFINITY, wy = INFINITY;
+    if (bb32) {
+        wx = ordered_to_flt(bb32[2]) - ordered_to_flt(bb32[0]);
+        wy = ordered_to_flt(bb32[3]) - ordered_to_flt(bb32[1]);
+    } else if (bbox) {
+        wx = (float)(ordered_to_dbl(bbox[1]) - ordered_to_dbl(bbox[0]));
+        wy = (float)(ordered_to_dbl(bbox[3]) - ordered_to_dbl(bbox[2]));
+    }
+    const float ext = fmaxf(wx, wy), ng = (float)P.n_groups;
+    const float per_d2 = (float)P.n_part / (kLocRho2 * rcm[0] * rcm[0]);  // stars near, over d^2
+    const bool narrow = ext < kNarrow * rcm[0], tiny = ext * rsqrtf(ng) < kTiny * rcm[0];
+    const bool dense = (bb32 || bbox) && wx * wy * (0.5f * kSuperGroups) * per_d2 > near_max * ng;
+    const int most_left = narrow ? (tiny ? kTinyLeft : -1) : dense ? -1 : kSuperLeft;
     for (;;) {
         uint32_t sg = 0;
         if (lane == 0) sg = atomicAdd(P.counter, 1u);
@@ -672,7 +696,7 @@ k_super(const __grid_constant__ WalkParams<float> P, const float* rcm, const uns
         float top2 = 0.0f;  // largest |alpha|^2 of one star left to the groups
         int sp = 1, left = 0, nf = 0, nn = 0;
         uint32_t work = 0;
-        bool ok = d < 1e30f;
+        bool ok = d < 1e30f && d * d * per_d2 <= 4.0f * near_max;
         // The buffers hold positions as the tree has them: the sums at the
         // centres subtract each group's own anchor, as its own walk does (the
         // subtraction is rounded: the anchor is part of the result's last digits).
@@ -861,7 +885,8 @@ k_super(const __grid_constant__ WalkParams<float> P, const float* rcm, const uns
 
 // Supergroups' records for the walk of a point-mass tree (null: not worth it).
 static const SuperRec* launch_super(WalkParams<float>& P, const SpeciesTree& st, char* base, const Layout& L,
-                                    uint32_t* counter, int64_t nb, int dtype, int num_sms, cudaStream_t s)
+                                    uint32_t* counter, int64_t nb, int dtype, float near_max, int num_sms,
+                                    cudaStream_t s)
 {
     constexpr size_t smem = kWalkWarps * sizeof(WalkShared<LENS_POINT, float, 0, 2>);
     static const int bps = [] {
@@ -878,7 +903,7 @@ static const SuperRec* launch_super(WalkParams<float>& P, const SpeciesTree& st,
     const int64_t blocks = std::min<int64_t>((ns + kWalkWarps - 1) / kWalkWarps, (int64_t)num_sms * bps);
     const void* box = base + L.bbox;  // of a single batch: ordered uint32 or FP64 images (enqueue_groups)
     k_super<<<(unsigned)blocks, kWalkWarps * 32, smem, s>>>(P, st.node_rcm, nb == 1 && dtype != LENS_F32 ? (const unsigned long long*)box : nullptr,
-                                                            nb == 1 && dtype == LENS_F32 ? (const uint32_t*)box : nullptr, rec, (float4*)(base + L.sdelta));
+                                                            nb == 1 && dtype == LENS_F32 ? (const uint32_t*)box : nullptr, near_max, rec, (float4*)(base + L.sdelta));
     note_launch();
     return rec;
 }
@@ -990,11 +1015,11 @@ static void launch_direct(int kind, bool ao, const WalkParams<T>& P, int num_sms
 // The one-warp tree walk of all groups.
 //   FP32 NFW trees (expansions) and, up to 4,096 groups, all but FP32 point
 //     masses: the cut form.
-//   FP32 point masses: the plain kernel with cuts (up to 16 groups per SM the
-//     cut form: more warps than that it can hold too, and its steps are shorter:
-//     504 groups of 67,587 stars 1.11 ms, 1.22; 1,501 of 1.6e6 1.85, 1.98).  With supergroups the cut form with
-//     expansions or, as only the device knows, the plain kernel: the other of
-//     the two launches finds no work.
+//   FP32 point masses: the plain kernel with cuts; up to 16 groups per SM (as
+//     many warps as either kernel has) the cut form, whose steps are shorter
+//     (504 groups of 67,587 stars 1.22 and 1.11 ms; 1,501 of 1.6e6 1.98, 1.85).
+//     With supergroups the cut form with expansions or, as only the device
+//     knows, the plain kernel: the other of the two launches finds no work.
 //   The others: from kPlainGroups groups on the stretched groups by the cut
 //     form and the rest by the plain kernel, whose 80 to 96 registers the cut
 //     form's 96 to 128 cost 5 to 10 %; below, all by the cut form, which cuts
@@ -1363,8 +1388,11 @@ static lens_status enqueue_typed(lens_tree* t, const ShootPlan& plan, const void
                 // the caller keeps no lists and counts nothing
                 if constexpr (sizeof(T) == 4) {
                     P.super = nullptr;
-                    if (st.kind == LENS_POINT && ng >= 16384 && !keep && !P.stats)
-                        P.super = launch_super(P, st, base, L, counter + 8 * launches + 3, nb, dtype, t->num_sms, s);
+                    if (st.kind == LENS_POINT && ng >= 16384 && !keep && !P.stats) {
+                        const double th = 0.3 / t->theta;
+                        P.super = launch_super(P, st, base, L, counter + 8 * launches + 3, nb, dtype,
+                                               R == 4 ? INFINITY : (float)(kNearMax * R * R * th * th * th), t->num_sms, s);
+                    }
                 }
                 P.counter = counter + 8 * launches;
                 if (R == 1) walk_tree<T, 1>(st.kind, ao, P, t, nq, base, L, s);

@@ -710,7 +710,7 @@ template <int KIND, typename T, int R, bool AO, int TILE, bool LOC> struct WalkF
                     bool point = true;
                     if constexpr (KIND != LENS_POINT) {
                         const float lo2 = kLocNear2 * r2;
-                        point = q.w <= 0.0f ? lo2 >= -q.w : KIND == LENS_GAUSS ? lo2 * q.w > S.ray.K.Uq : lo2 > q.w;
+                        point = q.w <= 0.0f ? lo2 >= -q.w : lo2 > q.w;
                     }
                     if (point && d * d * inv <= S.loc.rho2) {
                         direct = false;

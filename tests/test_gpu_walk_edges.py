@@ -236,3 +236,34 @@ def test_group_counts_at_the_rules(kind, groups):
         idx = np.unique(np.r_[0, rays - 1, g.integers(0, rays, 60)])
         _, absum = oracle.direct_sum(comps, dx[idx].astype(np.float64), dy[idx].astype(np.float64), with_absum=True)
         assert (np.abs(out[0][idx] - out[1][idx]) / (absum + 1e-300)).max() <= (1e-14 if prec == "fp64" else 1e-6)
+
+
+@pytest.mark.parametrize("width,group", [(1.3e-6, 128), (1.5e-6, 128), (0.0138, 64), (0.0144, 64), (0.9, 32), (1.6, 32), (1.6, 64)])
+@pytest.mark.parametrize("batches", [1, 2])
+def test_supergroup_rules(width, group, batches):
+    """Point masses over patches on both sides of the rules for supergroups: a
+    group's side an eighth of FP32's rounding, a patch 0.01 of the lens's
+    r_cm (1.41), fields with few and with many stars near a supergroup; as one
+    batch and as two, whose groups share a supergroup.  Reference: the
+    producer/consumer form, 1e-6 of the sum of |terms|."""
+    p = lensgen.point_disk(60_000, 55)
+    n = 1460 if group == 128 else 1030 if group == 64 else 760
+    dx, dy = lensgen.patch_offsets(n, width)
+    origin = (0.5, 0.01) if width < 1 else (0.0, 0.0)
+    assert dx.size >= 16384 * group
+    x, y, rays = cu(dx), cu(dy), dx.size
+    idx = np.unique(np.r_[0, rays - 1, lensgen.rng(3).integers(0, rays, 200)])
+    pick = torch.from_numpy(idx).cuda()
+    out = []
+    for walk in ("warp", "pairs"):
+        lens = L.Lens([L.Species.points(cu(p))], theta=0.3, group_rays=group, walk=walk)
+        if batches == 1:
+            o = lens.shoot(x, y, origin=origin)
+        else:
+            o = lens.shoot_batches(np.array([0, rays // 2 + 17, rays]), np.array([origin, origin]), x, y)
+        out.append(np.stack([v[pick].double().cpu().numpy() for v in o], 1))
+        lens.close()
+    rx, ry = origin[0] + dx[idx].astype(np.float64), origin[1] + dy[idx].astype(np.float64)
+    _, absum = oracle.direct_sum(comps_points(p), rx, ry, with_absum=True)
+    # (the reference groups at most 64 rays; over 1.5e-6 the decisions are the same)
+    assert (np.abs(out[0] - out[1]) / (absum + 1e-300)).max() <= 1e-6
