@@ -225,6 +225,12 @@ lens_status lens_build_tree(const lens_species* species, int32_t n_species,
  *       (4 B per entry: 2 KB per 32 rays, from cudaMalloc when they grow).
  *       A group whose lists exceed the room is marked and walked again by
  *       the adjoint.
+ *       With LENS_COUNT or LENS_KEEP_LISTS the walk of an FP32 tree of point
+ *       masses shares no expansions between ray groups (it does from 16,384
+ *       groups on): counts and lists are those of walks from the root, the
+ *       call takes longer, and the outputs may differ from those of the plain
+ *       call in their last digits.
+ * Repeated calls give the same bits (same rays, tree and flags).
  * A tree without particles (analytic components only) is shot one thread
  * per ray with no ray grouping, except with LENS_COUNT or LENS_TIMING, whose
  * counters and times refer to the grouped walk (the same terms either way).
@@ -482,9 +488,12 @@ lens_status lens_tree_export(const lens_tree* tree, int32_t s, void* nodes, int3
  *     [0] ray groups walked        [1] boxes visited (MAC evaluated)
  *     [2] cells accepted           [3] leaf particles evaluated
  *     [4] big-list entries scanned [5] big-list entries kept for a group
- *     [6] ray-interactions evaluated: sum over groups of rays x (cells +
- *         leaf particles + kept big entries)   [7] reserved (0)
- * Counts are per species launch and summed over species.
+ *     [6] ray-interactions: sum over groups of rays x (cells + leaf
+ *         particles + kept big entries)   [7] reserved (0)
+ * Counts are per species launch and summed over species.  FP32 NFW trees add
+ * most cells and leaf particles to one expansion per group instead of
+ * evaluating them for every ray: there [6] is the number of terms that the
+ * expansions stand for.
  */
 lens_status lens_tree_counters(lens_tree* tree, int64_t* out, int32_t reset);
 

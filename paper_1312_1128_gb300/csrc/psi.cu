@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(const __grid_const
                 C.flush_big();
                 if (P.n_halos > 0 && head && S.cut.seg == 0) C.halos();
                 // (a part's cut counts from its own start)
-                count_item(C, g, P.grange[g].y, head && S.cut.seg == 0);
+                count_item(C, g, head && S.cut.seg == 0);
                 C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
             } while (S.cut.local && local_next_part<R, 3>(P.cut, S.cut, stack, [&](int r, int q) {
                          return C.tot_s[r][q] + C.tot_c[r][q]; }));
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) psi_kernel(const __grid_const
         // (read again: kept in registers over the walk they cost it spills)
         if constexpr (!DIRECT) g = S.cut.g;
         const uint2 rg = P.grange[g];
-        if constexpr (FORM != 2) count_item(C, g, rg.y, head);
+        if constexpr (FORM != 2) count_item(C, g, head);
         T* tot = DIRECT ? nullptr : item_totals<R>(P.cut, S.cut);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -463,7 +463,7 @@ template <int KIND, typename T, int R, int FORM> static int psi_blocks_per_sm()
                                  (int)smem);
         int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psi_kernel<KIND, T, R, FORM>, kWalkWarps * 32, smem);
-        bps = std::min(std::max(nb, 1), FORM == 0 ? 16 : kWalkBlocks);  // (room for stacks and cuts)
+        bps = std::min(std::max(nb, 1), FORM == 0 ? 16 : walk_blocks<T, R>());  // (room for stacks and cuts)
     }
     return bps;
 }

@@ -437,14 +437,14 @@ walk_kernel(const __grid_constant__ WalkParams<T> P)
                 }
                 Ctx::Flush::finish(P.halos, first ? P.n_halos : 0, sr, delta);
                 // (a part's cut counts from its own start)
-                count_item(C, g, P.grange[g].y, first);
+                count_item(C, g, first);
                 C.c_vis = C.c_acc = C.c_near = C.c_bigs = C.c_bigk = 0;
             } while (S.cut.local && local_next_part<R, AO ? 2 : 5>(P.cut, S.cut, stack,
                                                                    [&](int r, int q) { return C.total(r, q); }));
         }
         __syncwarp();
         const uint2 rg = P.grange[g];
-        if constexpr (DIRECT) count_item(C, g, rg.y, head);
+        if constexpr (DIRECT) count_item(C, g, head);
 
         T* tot = DIRECT ? nullptr : item_totals<R>(P.cut, S.cut);
 #pragma unroll
@@ -541,7 +541,7 @@ walk_plain(const __grid_constant__ WalkParams<T> P)
                 ridx[r] = rv[r] ? P.ray_idx[rg.x + r * 32 + lane] : 0u;
             }
         }
-        count_item(C, kAgain ? S.cut.g : g, rg.y, true);
+        count_item(C, kAgain ? S.cut.g : g, true);
         if (CUTS && S.cut.sp > 0) cut_now<R, false>(P.cut, S.cut, stack, S.cut.sp);
         __syncwarp();
         T* tot = CUTS ? item_totals<R>(P.cut, S.cut) : nullptr;
@@ -574,8 +574,8 @@ template <int KIND, typename T, int R, bool AO, int TILE, bool CUTS> static int 
         cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kWalkWarps * 32, smem);
-        // (stacks are allocated for 16 blocks per SM; where cuts lie behind them: kWalkBlocks)
-        return std::min(std::max(nb, 1), CUTS ? kWalkBlocks : 16);
+        // (stacks are allocated for 16 blocks per SM; where cuts lie behind them: walk_blocks)
+        return std::min(std::max(nb, 1), CUTS ? walk_blocks<T, R>() : 16);
     }();
     return bps;
 }
@@ -962,7 +962,7 @@ static int walk_blocks_per_sm()
         int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, walk_kernel<KIND, T, R, AO, DIRECT, TILE, LOC>,
                                                       kWalkWarps * 32, smem);
-        cached = std::min(std::max(nb, 1), DIRECT ? 16 : kWalkBlocks);  // (room for stacks and cuts)
+        cached = std::min(std::max(nb, 1), DIRECT ? 16 : walk_blocks<T, R>());  // (room for stacks and cuts)
     }
     return cached;
 }
@@ -1018,9 +1018,10 @@ static void launch_direct(int kind, bool ao, const WalkParams<T>& P, int num_sms
 // The one-warp tree walk of all groups.
 //   FP32 NFW trees (expansions) and, up to 4,096 groups, all but FP32 point
 //     masses: the cut form.
-//   FP32 point masses: the plain kernel with cuts; up to 16 groups per SM (as
-//     many warps as either kernel has) the cut form, whose steps are shorter
-//     (504 groups of 67,587 stars 1.22 and 1.11 ms; 1,501 of 1.6e6 1.98, 1.85).
+//   FP32 point masses: the plain kernel with cuts; up to 32 groups per SM (about
+//     as many warps as it holds) the cut form, whose steps are shorter (504
+//     groups of 67,587 stars 1.22 and 1.11 ms; 2,793 of 2e6 2.01, 1.83; 4,278
+//     over a wide field of 1e6 1.12, 1.14; 14,964 1.33, 1.38).
 //     With supergroups the cut form with expansions or, as only the device
 //     knows, the plain kernel: the other of the two launches finds no work.
 //   The others: from kPlainGroups groups on the stretched groups by the cut
@@ -1056,7 +1057,7 @@ static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, co
         const int warps = std::max(cut_warps, kWalkWarps * sms * plain_blocks_per_sm<KIND, T, R, AO, TILE, true>());
         const bool fit = cuts_fit<T, R>(ng, L, warps, cut_warps);
         auto groups = [&](const WalkParams<T>& Q) {
-            const bool whole = fit && ng > 16 * sms;
+            const bool whole = fit && ng > 32 * sms;
             if (Q.super || !whole) cut(Q);
             if (!Q.super && !whole) return;
             WalkParams<T> W = Q;

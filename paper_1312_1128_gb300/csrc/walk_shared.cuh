@@ -52,11 +52,11 @@ struct Layout {
 
 // Cut groups (walk_dev.cuh): a call's cuts lie in the part of the stack region
 // that its launches leave unused (stacks are allocated for 16 blocks per SM, a
-// tree walk has at most kWalkBlocks: 80 MB and more are left), which
+// tree walk has at most walk_blocks(): 80 MB and more are left), which
 // walk_rounds splits: a place for each warp of the cut form, then two pools.
 // From about 600,000 rays on up to 48 MB are added behind it, so that every
 // group has a place in the first pool up to 24,576 groups.
-constexpr int kWalkBlocks = 8;
+template <typename T, int R> constexpr int walk_blocks() { return R * sizeof(T) > 8 ? 4 : 8; }
 constexpr size_t kCutSlotBytes = 2320;
 // Stretched groups: Morton order jumps between quadrants, so unless the rays
 // fill power-of-two squares a few groups span half the map and open most of

@@ -189,7 +189,7 @@ LENS_DEV void ws_produce(const WalkParams<T>& P, WsPair<KIND, T, CONS>& W, int* 
         C.handoff(kWsLast);
         if (!C.alive) return;
         if (C.rec && lane == 0) P.list_n[g] = whole && C.rec_n <= C.rec_cap ? (uint32_t)C.rec_n : kListTooLong;
-        count_item(C, g, P.grange[g].y, true);
+        count_item(C, g, true);
     }
 }
 
