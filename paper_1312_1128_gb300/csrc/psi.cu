@@ -570,7 +570,7 @@ static lens_status psi_typed(lens_tree* t, const ShootPlan& plan, const void* dx
                 // the cut form; small trees' whole groups by a kernel with 16 to
                 // 24 registers less (20,000 particles 1.04 to 1.2 times as fast;
                 // 300,000 particles, 25,992 groups 9.0 ms, the cut form 7.7)
-                const CutPlan cp{ng <= kFewGroups, false, false, 8};
+                const CutPlan cp{ng <= few_groups(kind, sizeof(T) == 4, P.n_part), false, false, 8};
                 const int cut_warps = psi_warps<T, R, 2>(kind, t->num_sms);
                 const int warps = std::max(cut_warps, psi_warps<T, R, 1>(kind, t->num_sms));
                 const bool cuts = cp.few || P.n_part >= 24576 || !cuts_fit<T, R>(ng, L, warps, cut_warps);

@@ -1016,8 +1016,8 @@ static void launch_direct(int kind, bool ao, const WalkParams<T>& P, int num_sms
 }
 
 // The one-warp tree walk of all groups.
-//   FP32 NFW trees (expansions) and, up to 4,096 groups, all but FP32 point
-//     masses: the cut form.
+//   FP32 NFW trees (expansions) and, where all groups are cut (few_groups), all
+//     but FP32 point masses: the cut form.
 //   FP32 point masses: the plain kernel with cuts; up to 32 groups per SM (about
 //     as many warps as it holds) the cut form, whose steps are shorter (504
 //     groups of 67,587 stars 1.22 and 1.11 ms; 2,793 of 2e6 2.01, 1.83; 4,278
@@ -1049,7 +1049,7 @@ static void walk_tree_kind(WalkParams<T> P, lens_tree* t, int nq, char* base, co
     };
     const int cut_warps = kWalkWarps * sms * (P.super ? walk_blocks_per_sm<KIND, T, R, AO, false, TILE, kPoint || kNfw>()
                                                       : walk_blocks_per_sm<KIND, T, R, AO, false, TILE, kNfw>());
-    const CutPlan plan{ng <= kFewGroups && !kPoint, kPoint, false};
+    const CutPlan plan{ng <= few_groups(KIND, kF32, P.n_part) && !kPoint, kPoint, false};
     if constexpr (kNfw) {
         if (never_cut(t, ng, P.n_rays, P.n_part, plan)) cut(P);
         else walk_rounds<T, R>(P, plan, nq, base, L, counter, cut, cut, cut_warps, cut_warps, s);

@@ -1516,10 +1516,17 @@ struct CutPlan {
     // deflection of 300,000 particles, 839^2 rays 7.3 ms, 16: 6.8)
     uint32_t heavy_parts = 16;
 };
-// Smaller trees gain up to here (20,000 particles, 4,072 groups 0.95 ms, as heavy
-// groups only 1.44; 100,000: 2.58, 3.03), larger ones less far (1e6 particles,
-// 512 groups and fewer; 1,287: 19.8, 8.2).
-constexpr int64_t kFewGroups = 4096;
+// Up to how many groups all are cut: 4,096, but 512 for FP32 Gaussian trees of
+// 200,000 particles and more.  Their groups' parts are heavy too and fill the
+// second pool.  Times with all groups cut, and with the heavy ones only: 20,000
+// particles, 4,072 groups 0.95 ms, 1.44; 60,000, 1,287: 1.02, 2.47; 100,000,
+// 1,800: 1.72, 1.55, 4,072: 2.58, 3.03; 300,000, 1,296 64-ray groups 11.0, 3.70
+// (without cuts 9.4), 4,072: 6.9, 3.2; 1e6, 1,287: 20.1, 8.2, 4,072: 15.5, 10.1;
+// potential, 300,000, 2,485: 8.4, 5.6; 1e6, 1,800: 5.6, 6.9 (the one that loses).
+inline int64_t few_groups(int kind, bool f32, int64_t n)
+{
+    return f32 && kind == LENS_GAUSS && n >= 200000 ? 512 : 4096;
+}
 
 // Is no group of a tree of n particles worth a cut (five more launches)?  Times
 // with cuts, and without, theta 0.3 (at smaller theta a walk meets more of a
@@ -1527,7 +1534,9 @@ constexpr int64_t kFewGroups = 4096;
 //   few groups: 400 particles, 100 to 1e5 rays 1.05 to 1.15 times as long; 700
 //     particles, 100 rays 0.22 ms, 0.29; FP64, 400 particles, 1,000 rays 0.59 ms,
 //     0.69.  Above 512 groups the groups are many beside the particles at first
-//     (3,750 groups, 1,200 particles 0.40 ms, 0.39; 5,000 particles 0.63, 0.81).
+//     (3,750 groups, 1,200 particles 0.40 ms, 0.39; 5,000 particles 0.63, 0.81;
+//     potential, 3,750 groups, 2,500 particles 0.64, 0.60; 2,329, 2,105: 0.47,
+//     0.53).
 //     One ray: 700 particles 0.126 ms, 0.100; 2,500 particles 0.113, 0.128.
 //   others: no walk is longer than 2 n + n / 16 entries (cells and leaf particles,
 //     listed ones, their tests), of point masses n; 0.3 ms for 16,384 entries.
@@ -1536,7 +1545,7 @@ inline bool never_cut(const lens_tree* t, int64_t ng, int64_t n_rays, int64_t n,
     const double th = std::min(t->theta / 0.3, 1.0);
     const int64_t small = t->precision == LENS_PREC_FP64 ? 256 : 512;
     if (plan.few)
-        return n <= th * (double)std::max(small, ng > 512 ? ng : 0) || (n_rays == 1 && n < 1024 * th * th);
+        return n <= th * (double)std::max(small, ng > 512 ? 7 * ng / 10 : 0) || (n_rays == 1 && n < 1024 * th * th);
     return plan.keep_order ? n < 8192 : 2 * n + n / 16 < 16384;
 }
 
@@ -1567,7 +1576,7 @@ template <typename T, int R> bool cuts_fit(int64_t ng, const Layout& L, int warp
 // kernel and their parts run in the next one; a part may be cut once more.
 // Launches without items cost about 3 us each, beside walks of 100 us and more.
 // warps: of the kernel with the most; cut_warps: of the cut form.
-//   few (up to 4,096 groups): about as many warps as the chip holds, or fewer.
+//   few (few_groups): about as many warps as the chip holds, or fewer.
 //     Up to 512 groups are cut as soon as their stack holds 64 boxes (their big
 //     lists deferred to the parts), into enough parts for about 8,192 warps; up
 //     to 4,096 after a share of work that about doubles the launch's warps.

@@ -267,3 +267,18 @@ def test_supergroup_rules(width, group, batches):
     _, absum = oracle.direct_sum(comps_points(p), rx, ry, with_absum=True)
     # (the reference groups at most 64 rays; over 1.5e-6 the decisions are the same)
     assert (np.abs(out[0] - out[1]) / (absum + 1e-300)).max() <= 1e-6
+
+
+@pytest.mark.parametrize("groups", [512, 513, 2500])
+def test_few_groups_of_a_large_tree(groups):
+    """Trees of 200,000 particles: all groups are cut up to 512 of them, heavy ones
+    above.  1e-6 of the sum of |terms|."""
+    from lens_testutil import comps_gauss
+    g = lensgen.rng(groups)
+    p = lensgen.nfw_particles(200_000, 7, nsph=32)
+    n = 32 * groups
+    dx, dy = (g.uniform(-0.9, 0.9, n).astype(np.float32) for _ in range(2))
+    got, ref = shoot([L.Species.gauss(cu(p), 3.0)], dx, dy), shoot([L.Species.gauss(cu(p), 3.0)], dx, dy, walk="pairs")
+    idx = np.unique(np.r_[0, n - 1, g.integers(0, n, 60)])
+    _, absum = oracle.direct_sum(comps_gauss(p, 3.0), dx[idx].astype(np.float64), dy[idx].astype(np.float64), with_absum=True)
+    assert (np.abs(got[idx] - ref[idx]) / (absum + 1e-300)).max() <= 1e-6
